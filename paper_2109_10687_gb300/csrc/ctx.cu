@@ -468,9 +468,11 @@ extern "C" int qcd_build_clover(qcd_ctx* ctx, void* stream) {
   ensure_alloc((void**)&ctx->cinv16, v * 36 * sizeof(__half2));
   cudaStream_t st = (cudaStream_t)stream;
   QCD_CUDA_CHECK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
+  ensure_alloc((void**)&ctx->udf, v * 36 * sizeof(float4));
+  ensure_alloc((void**)&ctx->clovdf, v * 36 * sizeof(float4));
+  sap_staging_alloc(ctx);
   build_clover_launch(ctx, st);
-  build_sap_staging(ctx, st);
-  build_df64_copies(ctx, true, true, st);
+  build_link_copies(ctx, st);
   int hs = 0;
   QCD_CUDA_CHECK(cudaMemcpyAsync(&hs, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
   QCD_CUDA_CHECK(cudaStreamSynchronize(st));

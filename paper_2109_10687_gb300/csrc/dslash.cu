@@ -768,35 +768,6 @@ void lat_dslash_df64_launch(const LatDesc* d_lat, const int* d_tile_lat, long lo
   check_launch();
 }
 
-// float64 (double2) fields -> double-float (float4) copies, elementwise, by
-// integer operations on the bits (links and clover entries are far inside
-// float32's range)
-__global__ void f64_to_df64_kernel(const double2* __restrict__ in, float4* out, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const double2 v = in[i];
-    const df64 re = df64_from_double_scaled(v.x, 0), im = df64_from_double_scaled(v.y, 0);
-    out[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
-  }
-}
-
-void build_df64_copies(qcd_ctx* ctx, bool links, bool clover, cudaStream_t st) {
-  const Geom& g = ctx->geom;
-  if (links) {
-    const size_t n = (size_t)g.vol * 36;
-    if (!ctx->udf) QCD_CUDA_CHECK(cudaMalloc(&ctx->udf, n * sizeof(float4)));
-    LaunchScope ls(ctx, QCD_KC_OTHER, st);
-    f64_to_df64_kernel<<<1024, 256, 0, st>>>(ctx->u64, ctx->udf, n);
-    check_launch();
-  }
-  if (clover) {
-    const size_t n = (size_t)g.vol * 36;
-    if (!ctx->clovdf) QCD_CUDA_CHECK(cudaMalloc(&ctx->clovdf, n * sizeof(float4)));
-    LaunchScope ls(ctx, QCD_KC_OTHER, st);
-    f64_to_df64_kernel<<<1024, 256, 0, st>>>(ctx->clov64, ctx->clovdf, n);
-    check_launch();
-  }
-}
-
 }  // namespace qcd
 
 using namespace qcd;

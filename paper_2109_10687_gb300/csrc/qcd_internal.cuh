@@ -791,8 +791,12 @@ void dslash_launch(qcd_ctx* ctx, void* out, const void* in, int prec, int mode, 
 void clover_apply_launch(qcd_ctx* ctx, void* out, const void* in, int prec, int inverse, int nrhs,
                          cudaStream_t st);
 void ablock_launch(qcd_ctx* ctx, float4* out, const float4* in, int row, int col, cudaStream_t st);
+// build_clover_launch writes every copy of 1 + C and its inverse and uses
+// ctx->udf as scratch; build_link_copies then writes the double-float links
+// there and the staged links of the SAP block kernel
 void build_clover_launch(qcd_ctx* ctx, cudaStream_t st);
-void build_sap_staging(qcd_ctx* ctx, cudaStream_t st);
+void build_link_copies(qcd_ctx* ctx, cudaStream_t st);
+void sap_staging_alloc(qcd_ctx* ctx);  // 4^4 domains only, else nothing
 bool sap_staged_available(const qcd_ctx* ctx);
 // halo: face halo of the shared-memory SAP kernel, 96 bytes per site and right-hand side
 void sap_staged_sequence_f32(qcd_ctx* ctx, F32Spinor s_first_in, F32Spinor s, F32Spinor x, F32Spinor b,
@@ -823,7 +827,6 @@ void gauge_import_launch(qcd_ctx* ctx, const double* u, cudaStream_t st);
 enum { MODE_D = 0, MODE_DDAG = 1, MODE_A = 2 };
 // internal precision code of the double-float operator (not part of the ABI)
 constexpr int PREC_DF64 = 7;
-void build_df64_copies(qcd_ctx* ctx, bool links, bool clover, cudaStream_t st);
 
 // one lattice of a ragged batch (device copy, rebuilt for every batched call)
 struct BatchDesc {
