@@ -10,21 +10,25 @@
 // (sigma_k (x) A = [[A_3, A_1 - i A_2], [A_1 + i A_2, -A_3]] on (spin, colour)),
 // each multiplied by i kappa c_SW.
 //
-// One block of the build kernel takes 32 sites in three phases: a warp per
-// plane computes F of its plane (a thread per site); a warp per chiral block
-// packs 1 + C and inverts it in float64; all six warps write every copy of
-// both that the library keeps, each a coalesced stream, from shared memory.
+// Two kernels: F of every site and plane (a thread each), then, a thread per
+// site and chiral block, 1 + C, its inverse in float64 and every copy of both
+// that the library keeps.  F waits in between in the buffer of 1 + C.
 //
-// What bounds it: this GPU has two float64 lanes per SM and cycle, and the
+// What bounds them: this GPU has two float64 lanes per SM and cycle, and the
 // leaves and inverses in float64 (11.2 k fused multiply-adds per site, one
 // thread per site) took 17.3 ms on 24^3 x 48, and the staging copies another
-// 0.64 ms; this kernel takes 5.4 ms for both.  Links of SU(3) are bounded by one, so their products are done
+// 0.64 ms.  Links of SU(3) are bounded by one, so their products are done
 // in fixed point instead, on the integer multipliers: a number is
 // (hi 2^29 + lo) 2^-58 with 30-bit signed hi and lo, a product of two is
 // three 32x32 -> 64 multiply-adds (lo lo, below 2^-59 of one, is left out),
 // and a sum of products stays in 64 bits.  The error of a matrix product is
 // a few units of 2^-58 of the entries' bound, below float64's 2^-53.
+// On 24^3 x 48 F takes 2.8 ms (the multipliers busy 55 %; 3.0 ms with 168
+// registers and 12 warps, 3.2 ms with 96 and 20) and the inversion 1.36 ms
+// (the float64 pipe busy 84 %).  One kernel with a barrier between the two
+// took 5.4 ms.
 
+#include "fixed.cuh"
 #include "qcd_internal.cuh"
 
 namespace qcd {
@@ -102,119 +106,12 @@ __device__ __noinline__ void field_strength(const Geom& g, const LinkPtr<double>
 }
 
 // ---------------------------------------------------------------------------
-// fixed-point 3x3 complex matrices
+// field strength
 // ---------------------------------------------------------------------------
-constexpr int FX_LIMB = 29;          // bits of the low limb
-constexpr int FX_FRAC = 2 * FX_LIMB; // a value is an integer times 2^-58
-
-struct FxMat {  // limbs of re and im, |hi| <= 2^30, |lo| <= 2^28
-  int rh[3][3], rl[3][3], ih[3][3], il[3][3];
-};
-struct FxSum {  // full 64-bit values
-  long long re[3][3], im[3][3];
-};
-
-// v = hi 2^29 + lo with lo rounded to the nearest
-__device__ __forceinline__ void fx_split(long long v, int& hi, int& lo) {
-  hi = (int)((v + (1LL << (FX_LIMB - 1))) >> FX_LIMB);
-  lo = (int)((unsigned)v - ((unsigned)hi << FX_LIMB));
-}
-__device__ __forceinline__ void fx_limbs(const FxSum& s, FxMat& m) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      fx_split(s.re[i][j], m.rh[i][j], m.rl[i][j]);
-      fx_split(s.im[i][j], m.ih[i][j], m.il[i][j]);
-    }
-}
-
-// float64 -> round(d 2^58), for |d| < 2^3, on the bit fields (the float64
-// pipe is the scarce one here)
-__device__ __forceinline__ long long fx_from_double(double d) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-  const int e = (int)((b >> 52) & 0x7FF);
-  if (e == 0) return 0;
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int sh = e - 1023 - 52 + FX_FRAC;  // value = m 2^sh units
-  unsigned long long v;
-  if (sh >= 0) v = m << sh;
-  else if (sh > -54) v = (m + (1ull << (-sh - 1))) >> -sh;
-  else v = 0;
-  return (b >> 63) ? -(long long)v : (long long)v;
-}
-
-// C = op(A) op(B), op the conjugate transpose where DA / DB is set.  Sums of
-// six products of |hi| <= 2^29 and 2^30 stay below 2^62.
-template <bool DA, bool DB>
-__device__ __forceinline__ void fx_mul(const FxMat& A, const FxMat& B, FxSum& C) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    // this row's real parts, imaginary parts, and the two operands whose
-    // sign the complex product flips (re: -ai bi, im: +ar bi, with bi -> -bi for DB)
-    int ah[3], al[3], bh[3], bl[3], ph[3], pl[3], qh[3], ql[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      ah[k] = DA ? A.rh[k][i] : A.rh[i][k];
-      al[k] = DA ? A.rl[k][i] : A.rl[i][k];
-      const int xh = DA ? A.ih[k][i] : A.ih[i][k], xl = DA ? A.il[k][i] : A.il[i][k];
-      bh[k] = DA ? -xh : xh;
-      bl[k] = DA ? -xl : xl;
-      ph[k] = DB ? bh[k] : -bh[k];
-      pl[k] = DB ? bl[k] : -bl[k];
-      qh[k] = DB ? -ah[k] : ah[k];
-      ql[k] = DB ? -al[k] : al[k];
-    }
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      long long rh = 0, rx = 1LL << (FX_LIMB - 1), ih = 0, ix = 1LL << (FX_LIMB - 1);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const int yrh = DB ? B.rh[j][k] : B.rh[k][j], yrl = DB ? B.rl[j][k] : B.rl[k][j];
-        const int yih = DB ? B.ih[j][k] : B.ih[k][j], yil = DB ? B.il[j][k] : B.il[k][j];
-        rh += (long long)ah[k] * yrh;
-        rh += (long long)ph[k] * yih;
-        rx += (long long)ah[k] * yrl;
-        rx += (long long)al[k] * yrh;
-        rx += (long long)ph[k] * yil;
-        rx += (long long)pl[k] * yih;
-        ih += (long long)qh[k] * yih;
-        ih += (long long)bh[k] * yrh;
-        ix += (long long)qh[k] * yil;
-        ix += (long long)ql[k] * yih;
-        ix += (long long)bh[k] * yrl;
-        ix += (long long)bl[k] * yrh;
-      }
-      C.re[i][j] = rh + (rx >> FX_LIMB);
-      C.im[i][j] = ih + (ix >> FX_LIMB);
-    }
-  }
-}
-
-// A -= B^dag
-__device__ __forceinline__ void fx_sub_dag(FxSum& A, const FxSum& B) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      A.re[i][j] -= B.re[j][i];
-      A.im[i][j] += B.im[j][i];
-    }
-}
-// A -= B
-__device__ __forceinline__ void fx_sub(FxSum& A, const FxSum& B) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      A.re[i][j] -= B.re[i][j];
-      A.im[i][j] -= B.im[i][j];
-    }
-}
-
-// links as limbs, int4 (re hi, re lo, im hi, im lo) [dom][mu][9][vd]
+// The link of direction dir at x + dm e_mu + dn e_nu, or its adjoint, from
+// limbs stored as int4 (re hi, re lo, im hi, im lo) [dom][mu][9][vd]
 __device__ __forceinline__ FxMat fx_link(const Geom& g, const int4* __restrict__ U, const int x[4], int mu, int nu,
-                                         int dm, int dn, int dir) {
+                                         int dm, int dn, int dir, bool dag) {
   int y[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -224,63 +121,87 @@ __device__ __forceinline__ FxMat fx_link(const Geom& g, const int4* __restrict__
   int dom, s;
   coords_to_internal(g, y, dom, s);
   const int4* p = U + (((size_t)((dom * 4 + dir) * 9)) << g.logvd) + s;
+  const int row = dag ? 1 : 3, col = dag ? 3 : 1, sg = dag ? -1 : 0;
   FxMat m;
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    const int4 v = __ldg(p + ((size_t)e << g.logvd));
-    m.rh[e / 3][e % 3] = v.x;
-    m.rl[e / 3][e % 3] = v.y;
-    m.ih[e / 3][e % 3] = v.z;
-    m.il[e / 3][e % 3] = v.w;
-  }
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int4 v = __ldg(p + ((size_t)(i * row + j * col) << g.logvd));
+      m.rh[i][j] = v.x;
+      m.rl[i][j] = v.y;
+      m.ih[i][j] = (v.z ^ sg) - sg;
+      m.il[i][j] = (v.w ^ sg) - sg;
+    }
   return m;
 }
 
 // F_mu,nu at x, as its nine independent reals: the imaginary parts of the
-// diagonal, then (re, im) of the entries 01, 02, 12.  Two leaves share a
-// first factor and two a last one up to the conjugate transpose, and only
-// Q - Q^dag is needed:
-//   Q - Q^dag = M - M^dag,  M = U_mu(n) (A - B^dag) + (C - E) U_mu(n - mu),
-// with A, B^dag, C, E products of three links: ten matrix products instead
-// of twelve.
+// diagonal, then (re, im) of the entries 01, 02, 12.  Only Q - Q^dag is
+// needed, so a leaf may be replaced by minus its adjoint, and the four leaves
+// pair up by their first factor:
+//   Q - Q^dag = M - M^dag,  M = sum_h L (X - Y^dag)  over two halves h,
+// X and Y products of three links: ten matrix products instead of twelve.
+// Both halves and both triple products are loops over the same code, whose
+// instructions then fit the cache; X waits in shared memory (stash, this
+// thread's column of a [18][FS_THREADS] array) while Y is formed.
+constexpr int FS_THREADS = 128;
+struct PathLink {  // direction (0 mu, 1 nu), offsets along mu and nu, adjoint
+  signed char dir, dm, dn, dag;
+};
+// [half]: X's three links, Y's three, L
+__constant__ PathLink c_path[2][7] = {
+    {{1, 1, 0, 0}, {0, 0, 1, 1}, {1, 0, 0, 1}, {1, 0, -1, 1}, {0, 0, -1, 0}, {1, 1, -1, 0}, {0, 0, 0, 0}},
+    {{1, -1, -1, 1}, {0, -1, -1, 0}, {1, 0, -1, 0}, {1, 0, 0, 0}, {0, -1, 1, 1}, {1, -1, 0, 1}, {0, -1, 0, 1}},
+};
 __device__ __forceinline__ void field_strength_fx(const Geom& g, const int4* U, const int x[4], int mu, int nu,
-                                                  double f[9]) {
-  auto at = [&](int dm, int dn, int dir) { return fx_link(g, U, x, mu, nu, dm, dn, dir); };
-  FxSum M, S, T;
-  FxMat t;
-  {  // A - B^dag, with U_nu(n) and then U_nu(n - nu) as the outer factor
-    fx_mul<false, true>(at(1, 0, nu), at(0, 1, mu), S);
-    fx_limbs(S, t);
-    fx_mul<false, true>(t, at(0, 0, nu), S);
-    fx_mul<false, false>(at(0, -1, mu), at(1, -1, nu), T);
-    fx_limbs(T, t);
-    fx_mul<true, false>(at(0, -1, nu), t, T);
-    fx_sub_dag(S, T);
-    fx_limbs(S, t);
-    fx_mul<false, false>(at(0, 0, mu), t, M);
-  }
-  {  // C - E
-    fx_mul<false, true>(at(0, 0, nu), at(-1, 1, mu), S);
-    fx_limbs(S, t);
-    fx_mul<false, true>(t, at(-1, 0, nu), S);
-    fx_mul<true, false>(at(-1, -1, mu), at(-1, -1, nu), T);
-    fx_limbs(T, t);
-    fx_mul<true, false>(at(0, -1, nu), t, T);
-    fx_sub(S, T);
-    fx_limbs(S, t);
-    fx_mul<false, false>(t, at(-1, 0, mu), S);
+                                                  long long* stash, double f[9]) {
+  long long acc[9];
+#pragma unroll
+  for (int e = 0; e < 9; ++e) acc[e] = 0;
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    auto link = [&](int k) {
+      const PathLink q = c_path[h][k];
+      return fx_link(g, U, x, mu, nu, q.dm, q.dn, q.dir ? nu : mu, q.dag != 0);
+    };
+    FxSum P;
+    FxMat t;
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+      fx_mul(link(3 * q), link(3 * q + 1), P);
+      fx_limbs(P, t);
+      fx_mul(t, link(3 * q + 2), P);
+      if (q == 0) {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+          stash[2 * e * FS_THREADS] = P.re[e / 3][e % 3];
+          stash[(2 * e + 1) * FS_THREADS] = P.im[e / 3][e % 3];
+        }
+      }
+    }
+    FxSum D;  // X - Y^dag
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      D.re[e / 3][e % 3] = stash[2 * e * FS_THREADS] - P.re[e % 3][e / 3];
+      D.im[e / 3][e % 3] = stash[(2 * e + 1) * FS_THREADS] + P.im[e % 3][e / 3];
+    }
+    fx_limbs(D, t);
+    fx_mul(link(6), t, P);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) acc[i] += 2 * P.im[i][i];
+    int o = 3;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = i + 1; j < 3; ++j) {
+        acc[o++] += P.re[i][j] - P.re[j][i];
+        acc[o++] += P.im[i][j] + P.im[j][i];
+      }
   }
   const double u = 1.0 / (double)(1LL << FX_FRAC) / 8.0;  // a power of two
 #pragma unroll
-  for (int i = 0; i < 3; ++i) f[i] = u * (double)(2 * (M.im[i][i] + S.im[i][i]));
-  int o = 3;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = i + 1; j < 3; ++j) {
-      f[o++] = u * (double)((M.re[i][j] + S.re[i][j]) - (M.re[j][i] + S.re[j][i]));
-      f[o++] = u * (double)((M.im[i][j] + S.im[i][j]) + (M.im[j][i] + S.im[j][i]));
-    }
+  for (int e = 0; e < 9; ++e) f[e] = u * (double)acc[e];
 }
 
 // inverse by Gauss-Jordan with partial pivoting, for blocks that are not
@@ -371,9 +292,9 @@ __device__ __forceinline__ bool invert6_packed(double m[36]) {
   return ok;
 }
 
-// the same through the pivoted elimination, from r to out (element k at
+// the same through the pivoted elimination, in place (element k at
 // k stride; zero if singular)
-__device__ __noinline__ bool invert6_general(const double* r, double* out, int stride) {
+__device__ __noinline__ bool invert6_general(double* r, int stride) {
   C64 m[6][6], inv[6][6];
   for (int i = 0; i < 6; ++i) {
     m[i][i] = make_cx(r[i * stride], 0.0);
@@ -385,11 +306,11 @@ __device__ __noinline__ bool invert6_general(const double* r, double* out, int s
   }
   const bool ok = invert6(m, inv);
   for (int i = 0; i < 6; ++i) {
-    out[i * stride] = ok ? inv[i][i].re : 0.0;
+    r[i * stride] = ok ? inv[i][i].re : 0.0;
     for (int j = i + 1; j < 6; ++j) {
       const int o = 6 + 2 * herm_off(i, j);
-      out[o * stride] = ok ? 0.5 * (inv[i][j].re + inv[j][i].re) : 0.0;
-      out[(o + 1) * stride] = ok ? 0.5 * (inv[i][j].im - inv[j][i].im) : 0.0;
+      r[o * stride] = ok ? 0.5 * (inv[i][j].re + inv[j][i].re) : 0.0;
+      r[(o + 1) * stride] = ok ? 0.5 * (inv[i][j].im - inv[j][i].im) : 0.0;
     }
   }
   return ok;
@@ -438,13 +359,8 @@ __device__ __forceinline__ void pack_block(const F& f, int b, double kc, double 
 }
 
 // ---------------------------------------------------------------------------
-// the build kernel
+// the kernels
 // ---------------------------------------------------------------------------
-constexpr int CB_SITES = 32;
-constexpr int CB_THREADS = 6 * CB_SITES;  // a warp per plane
-constexpr int CB_STRIDE = CB_SITES + 1;   // an odd stride: rows and columns without bank conflicts
-constexpr size_t CB_SMEM = sizeof(double) * (54 + 144) * CB_STRIDE + sizeof(size_t) * CB_SITES;
-
 struct CloverOut {
   double2 *clov64, *cinv64;   // [dom][36][vd]
   float4 *clov32, *cinv32;    // [dom][18][vd]
@@ -454,99 +370,135 @@ struct CloverOut {
   float4* st32;               // [dom][site][19]
 };
 
+// F between the kernels: a plane's nine reals in five double2 (the last half
+// filled), component 5 plane + k of [dom][36][vd] -- each site's own entries
+// of the buffer that 1 + C overwrites
+constexpr int F_PAIRS = 5;
+
+// A warp takes 32 consecutive sites (in lexicographic-domain order, so that
+// neighbouring domains' links are still in L2) and one plane; the six planes
+// of a tile are consecutive warps and share its links through L1.  No
+// barrier and 128 registers: 16 warps per SM keep the multipliers busy
+// (phases of one fused kernel, with 12 warps and its barriers, left them
+// two thirds idle).
 template <bool FIXED>
-__global__ void __launch_bounds__(CB_THREADS, 2) clover_build_kernel(Geom g, const int4* __restrict__ ufx,
-                                                                     LinkPtr<double> U, double kc, CloverOut o,
-                                                                     int* status) {
-  extern __shared__ double csm[];
-  double* sf = csm;                         // F: [plane][9][site]
-  double* sm = csm + 54 * CB_STRIDE;        // 1 + C, then its inverse: [2][block][36][site]
-  size_t* sbase = reinterpret_cast<size_t*>(sm + 144 * CB_STRIDE);  // (dom, s) of every site
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__global__ void __launch_bounds__(FS_THREADS, 4) field_strength_kernel(Geom g, const int4* __restrict__ ufx,
+                                                                       LinkPtr<double> U, double2* out) {
+  __shared__ long long stash[FIXED ? 18 * FS_THREADS : 1];
+  const int lane = threadIdx.x & 31;
+  const long long item = blockIdx.x * (long long)(FS_THREADS / 32) + (threadIdx.x >> 5);
+  const int p = (int)(item % 6);
+  const long long gid = item / 6 * 32 + lane;
+  if (gid >= g.vol) return;
+  int x[4], lex = (int)(gid >> g.logvd);
+  const int s = (int)(gid & (g.vd - 1));
+  const int dom = __ldg(g.lex2dom + lex);
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    const int q = lex / g.nd[mu];
+    x[mu] = (lex - q * g.nd[mu]) * g.d[mu] + ((s >> g.shift[mu]) & (g.d[mu] - 1));
+    lex = q;
+  }
+  const int mu = p < 3 ? 0 : (p < 5 ? 1 : 2);
+  const int nu = p < 3 ? p + 1 : (p < 5 ? p - 1 : 3);
+  double f[10];
+  f[9] = 0.0;
+  if (FIXED) field_strength_fx(g, ufx, x, mu, nu, stash + threadIdx.x, f);
+  else field_strength(g, U, x, mu, nu, f);
+#pragma unroll
+  for (int k = 0; k < F_PAIRS; ++k)
+    out[(((size_t)(dom * 36 + F_PAIRS * p + k)) << g.logvd) + s] = make_double2(f[2 * k], f[2 * k + 1]);
+}
+
+// float64 rounded to float32 on the bit fields (conversions would queue on
+// the float64 pipe; results below float32's normal range become zero)
+__device__ __forceinline__ float to_float(double d) { return df64_from_double_scaled(d, 0).hi; }
+
+// Threads (site, block): warps 0 and 1 the two blocks of 32 sites, warps 2
+// and 3 those of the next 32.  The float64 pipe bounds it (the inversion);
+// every component it writes is one stream over the warp's sites, only the
+// site-major staging rows go through shared memory.
+constexpr int CB_THREADS = 128;
+constexpr int CB_SITES = CB_THREADS / 2;
+constexpr int CB_ROW = 73;  // floats per site in shared memory, odd: no bank conflicts
+__global__ void __launch_bounds__(CB_THREADS, 4) clover_build_kernel(Geom g, double kc, CloverOut o, int* status) {
+  __shared__ float stage[CB_SITES * CB_ROW];
+  __shared__ double rows[36 * CB_THREADS];  // the pivoted inversion's operand and result
+  const int b = (threadIdx.x >> 5) & 1;
+  const int local = (threadIdx.x & 31) + (threadIdx.x >> 6) * 32;
   const long long n0 = blockIdx.x * (long long)CB_SITES;
-  const int live = (int)min((long long)CB_SITES, g.vol - n0);
+  const bool live = n0 + local < g.vol;
+  const long long gid = live ? n0 + local : n0;
+  const int dom = (int)(gid >> g.logvd), s = (int)(gid & (g.vd - 1));
+  const size_t at = ((size_t)dom * 36 << g.logvd) + s;
+  double m[36];
   {
-    // sites in lexicographic-domain order, so that neighbouring domains'
-    // links are still in L2; a block's sites past the end repeat its first
-    const long long gid = n0 + (lane < live ? lane : 0);
-    int x[4], lex = (int)(gid >> g.logvd);
-    const int s = (int)(gid & (g.vd - 1));
+    double f[60];
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      const int q = lex / g.nd[mu];
-      x[mu] = (lex - q * g.nd[mu]) * g.d[mu] + ((s >> g.shift[mu]) & (g.d[mu] - 1));
-      lex = q;
+    for (int k = 0; k < 6 * F_PAIRS; ++k) {
+      const double2 v = o.clov64[at + ((size_t)k << g.logvd)];
+      f[2 * k] = v.x;
+      f[2 * k + 1] = v.y;
     }
-    if (warp == 0) sbase[lane] = ((size_t)__ldg(g.lex2dom + (int)(gid >> g.logvd)) << 8) | (size_t)s;
-    const int mu = warp < 3 ? 0 : (warp < 5 ? 1 : 2);
-    const int nu = warp < 3 ? warp + 1 : (warp < 5 ? warp - 1 : 3);
-    double f[9];
-    if (FIXED) field_strength_fx(g, ufx, x, mu, nu, f);
-    else field_strength(g, U, x, mu, nu, f);
-#pragma unroll
-    for (int e = 0; e < 9; ++e) sf[(warp * 9 + e) * CB_STRIDE + lane] = f[e];
+    pack_block([&](int p, int e) { return f[2 * F_PAIRS * p + e]; }, b, kc, m);
   }
-  __syncthreads();
-  if (warp < 2) {
-    double m[36];
-    pack_block([&](int p, int e) { return sf[(p * 9 + e) * CB_STRIDE + lane]; }, warp, kc, m);
-    double* out = sm + warp * 36 * CB_STRIDE + lane;
+  __syncthreads();  // every F of the block is read before 1 + C overwrites it
+  if (live) {
 #pragma unroll
-    for (int k = 0; k < 36; ++k) out[k * CB_STRIDE] = m[k];
-    double* inv = out + 72 * CB_STRIDE;
-    bool ok = invert6_packed(m);
-#pragma unroll
-    for (int k = 0; k < 36; ++k) inv[k * CB_STRIDE] = m[k];
-    if (!ok) ok = invert6_general(out, inv, CB_STRIDE);
-    bool finite = true;
-    for (int k = 0; k < 36; ++k) finite = finite && isfinite(inv[k * CB_STRIDE]);
-    if ((!ok || !finite) && lane < live) atomicExch(status, 1);
-  }
-  __syncthreads();
-  // every copy; lane = site: each component is one stream over the sites
-  if (lane < live) {
-    const size_t base = sbase[lane];
-    const size_t dom = base >> 8, s = base & 255;
-    const double* v = sm + lane;
-    for (int k = warp; k < 36; k += 6) {
-      const size_t i = ((dom * 36 + k) << g.logvd) + s;
-      const double c0 = v[2 * k * CB_STRIDE], c1 = v[(2 * k + 1) * CB_STRIDE];
-      const double q0 = v[(72 + 2 * k) * CB_STRIDE], q1 = v[(73 + 2 * k) * CB_STRIDE];
-      o.clov64[i] = make_double2(c0, c1);
-      o.cinv64[i] = make_double2(q0, q1);
-      o.cinv16[i] = __floats2half2_rn((float)q0, (float)q1);
-      const df64 d0 = df64_from_double_scaled(c0, 0), d1 = df64_from_double_scaled(c1, 0);
+    for (int k = 0; k < 18; ++k) {
+      const size_t i = at + ((size_t)(18 * b + k) << g.logvd);
+      o.clov64[i] = make_double2(m[2 * k], m[2 * k + 1]);
+      const df64 d0 = df64_from_double_scaled(m[2 * k], 0), d1 = df64_from_double_scaled(m[2 * k + 1], 0);
       o.clovdf[i] = make_float4(d0.hi, d0.lo, d1.hi, d1.lo);
     }
-    for (int k = warp; k < 18; k += 6) {
-      const size_t i = ((dom * 18 + k) << g.logvd) + s;
-      const double* c = v + 4 * k * CB_STRIDE;
-      const double* q = c + 72 * CB_STRIDE;
-      o.clov32[i] = make_float4((float)c[0], (float)c[CB_STRIDE], (float)c[2 * CB_STRIDE], (float)c[3 * CB_STRIDE]);
-      o.cinv32[i] = make_float4((float)q[0], (float)q[CB_STRIDE], (float)q[2 * CB_STRIDE], (float)q[3 * CB_STRIDE]);
-    }
-  }
-  if (o.st16) {
-    // 4^4 domains: the 32 sites are consecutive sites of one domain, and so
-    // is their stretch of the site-major staging layouts
-    const size_t site0 = (sbase[0] >> 8) * 256 + (sbase[0] & 255);
-    for (int i = threadIdx.x; i < CB_SITES * 9; i += CB_THREADS) {
-      const double* q = sm + (size_t)(72 + 8 * (i % 9)) * CB_STRIDE + i / 9;
-      __half2 h[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        h[e] = __floats2half2_rn((float)q[2 * e * CB_STRIDE], (float)q[(2 * e + 1) * CB_STRIDE]);
-      o.st16[site0 * 9 + i] = *reinterpret_cast<const uint4*>(h);
+    for (int k = 0; k < 9; ++k)
+      o.clov32[((size_t)(dom * 18 + 9 * b + k) << g.logvd) + s] =
+          make_float4(to_float(m[4 * k]), to_float(m[4 * k + 1]), to_float(m[4 * k + 2]), to_float(m[4 * k + 3]));
+  }
+  double* row = rows + threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < 36; ++k) row[k * CB_THREADS] = m[k];
+  bool ok = invert6_packed(m);
+  if (!ok) {
+    ok = invert6_general(row, CB_THREADS);
+#pragma unroll
+    for (int k = 0; k < 36; ++k) m[k] = row[k * CB_THREADS];
+  }
+  bool finite = true;
+#pragma unroll
+  for (int k = 0; k < 36; ++k) finite = finite && isfinite(m[k]);
+  if (live && !(ok && finite)) atomicExch(status, 1);
+  float* st = stage + local * CB_ROW + 36 * b;
+  if (live) {
+#pragma unroll
+    for (int k = 0; k < 18; ++k) {
+      const size_t i = at + ((size_t)(18 * b + k) << g.logvd);
+      const float q0 = to_float(m[2 * k]), q1 = to_float(m[2 * k + 1]);
+      o.cinv64[i] = make_double2(m[2 * k], m[2 * k + 1]);
+      o.cinv16[i] = __floats2half2_rn(q0, q1);
+      st[2 * k] = q0;
+      st[2 * k + 1] = q1;
     }
-    for (int i = threadIdx.x; i < CB_SITES * 19; i += CB_THREADS) {
-      const int k = i % 19;
-      float4 w = make_float4(0.f, 0.f, 0.f, 0.f);  // the last one pads the site
-      if (k < 18) {
-        const double* q = sm + (size_t)(72 + 4 * k) * CB_STRIDE + i / 19;
-        w = make_float4((float)q[0], (float)q[CB_STRIDE], (float)q[2 * CB_STRIDE], (float)q[3 * CB_STRIDE]);
-      }
-      o.st32[site0 * 19 + i] = w;
-    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+      o.cinv32[((size_t)(dom * 18 + 9 * b + k) << g.logvd) + s] =
+          make_float4(st[4 * k], st[4 * k + 1], st[4 * k + 2], st[4 * k + 3]);
+  }
+  if (!o.st16) return;
+  // 4^4 domains: every block is full, its sites are consecutive sites of one
+  // domain, and so are their rows in the staging layouts
+  __syncthreads();
+  for (int i = threadIdx.x; i < CB_SITES * 9; i += CB_THREADS) {
+    const float* q = stage + i / 9 * CB_ROW + 8 * (i % 9);
+    __half2 h[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(q[2 * e], q[2 * e + 1]);
+    o.st16[n0 * 9 + i] = *reinterpret_cast<const uint4*>(h);
+  }
+  for (int i = threadIdx.x; i < CB_SITES * 19; i += CB_THREADS) {
+    const float* q = stage + i / 19 * CB_ROW + 4 * (i % 19);
+    o.st32[n0 * 19 + i] = i % 19 < 18 ? make_float4(q[0], q[1], q[2], q[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
@@ -565,19 +517,10 @@ __global__ void links_to_fixed_kernel(const double2* __restrict__ u64, int4* out
 // switching that check off, take the float64 products.
 void build_clover_launch(qcd_ctx* ctx, cudaStream_t st) {
   const Geom& g = ctx->geom;
-  static const bool attr = [] {
-    QCD_CUDA_CHECK(cudaFuncSetAttribute(clover_build_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)CB_SMEM));
-    QCD_CUDA_CHECK(cudaFuncSetAttribute(clover_build_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)CB_SMEM));
-    return true;
-  }();
-  (void)attr;
   const CloverOut o{ctx->clov64, ctx->cinv64, ctx->clov32, ctx->cinv32, ctx->cinv16, ctx->clovdf,
                     (uint4*)ctx->st_clov16, (float4*)ctx->st_clov32};
-  const int grid = grid_for(g.vol, CB_SITES);
+  const int grid = grid_for((g.vol + 31) / 32 * 6, FS_THREADS / 32);
   const LinkPtr<double> U{ctx->u64};
-  const double kc = ctx->kappa * ctx->csw;
   if (ctx->su3_links) {
     // the limbs lie where the double-float links go once the clover term is built
     int4* ufx = reinterpret_cast<int4*>(ctx->udf);
@@ -587,13 +530,16 @@ void build_clover_launch(qcd_ctx* ctx, cudaStream_t st) {
       check_launch();
     }
     LaunchScope ls(ctx, QCD_KC_OTHER, st);
-    clover_build_kernel<true><<<grid, CB_THREADS, CB_SMEM, st>>>(g, ufx, U, kc, o, ctx->d_status);
+    field_strength_kernel<true><<<grid, FS_THREADS, 0, st>>>(g, ufx, U, ctx->clov64);
     check_launch();
   } else {
     LaunchScope ls(ctx, QCD_KC_OTHER, st);
-    clover_build_kernel<false><<<grid, CB_THREADS, CB_SMEM, st>>>(g, nullptr, U, kc, o, ctx->d_status);
+    field_strength_kernel<false><<<grid, FS_THREADS, 0, st>>>(g, nullptr, U, ctx->clov64);
     check_launch();
   }
+  LaunchScope ls(ctx, QCD_KC_OTHER, st);
+  clover_build_kernel<<<grid_for(g.vol, CB_SITES), CB_THREADS, 0, st>>>(g, ctx->kappa * ctx->csw, o, ctx->d_status);
+  check_launch();
 }
 
 }  // namespace qcd

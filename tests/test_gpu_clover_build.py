@@ -1,4 +1,5 @@
-"""The clover build kernel against the oracle, where its paths can go wrong.
+"""The gauge import and the clover build kernels against the oracle, where their
+paths can go wrong.
 
 1 + C and its inverse in float64 (through qcd_apply_clover) on lattices with
 fewer sites than a block, with storage blocks smaller and larger than a warp,
@@ -48,5 +49,49 @@ def test_clover_and_inverse(dims, domain, csw, scale):
         assert _rel(lat.apply_clover(psi, "double", inverse=True), op.apply_cinv(psi)) <= 2e-15 * max(10.0, cond)
         assert _rel(lat.apply_clover(psi, "single"), site_mul(m, psi)) <= 1e-6
         assert _rel(lat.apply_D(psi, "double"), op.D(psi)) <= 1e-14
+    finally:
+        lat.close()
+
+
+@pytest.mark.parametrize("dims,domain", [((2, 2, 2, 2), (1, 1, 1, 1)), ((4, 4, 8, 12), (2, 1, 2, 2)),
+                                         ((8, 8, 8, 8), (4, 4, 4, 4))])
+@pytest.mark.parametrize("delta", [3e-13, 2e-9, 0.03, 0.5, 3.0])
+def test_su3_check_reports_the_deviation(dims, domain, delta):
+    """set_gauge's message gives the worst |Re| + |Im| of U^dag U - 1 and det U - 1:
+    one link off by delta, in the fixed-point range and beyond it."""
+    from paper_2109_10687_gb300 import binding as B
+    from paper_2109_10687_gb300.lattice import Lattice
+
+    u = random_su3_field(dims, 0.6, 4003)
+    link = u[-1, 0, -1, 1, 2]
+    link[1, 2] += delta * (1 - 0.5j)
+    w = link.conj().T @ link - np.eye(3)
+    det = np.linalg.det(link) - 1
+    want = max((np.abs(w.real) + np.abs(w.imag)).max(), abs(det.real) + abs(det.imag))
+    lat = Lattice(dims, domain, -1, "chiral")
+    try:
+        with pytest.raises(B.QcdError) as e:
+            lat.set_gauge(u, check_tol=1e-13)
+        got = float(str(e.value).split("SU(3) by ")[1].split()[0])
+        # printed with four digits; the generated links are SU(3) to about 2e-15
+        assert abs(got - want) <= 1e-3 * want + 4e-15
+        lat.set_gauge(u, check_tol=2 * want)  # and what lies within the tolerance is taken
+    finally:
+        lat.close()
+
+
+def test_non_finite_links_are_refused_by_the_clover_build():
+    from paper_2109_10687_gb300 import binding as B
+    from paper_2109_10687_gb300.lattice import Lattice
+
+    u = random_su3_field((8, 8, 8, 8), 0.3, 4004)
+    u[3, 2, 1, 5, 0, 1, 1] = np.nan
+    lat = Lattice((8, 8, 8, 8), (4, 4, 4, 4), -1, "chiral")
+    try:
+        lat.set_gauge(u, check_tol=0.0)
+        lat.set_params(0.12, 1.0)
+        with pytest.raises(B.QcdError) as e:
+            lat.build_clover()
+        assert e.value.code == B.QCD_ERR_NONFINITE
     finally:
         lat.close()
