@@ -701,7 +701,6 @@ struct qcd_ctx {
   void* st_clov16 = nullptr;
   void* st_clov32 = nullptr;
   int* flow_state = nullptr;       // one-launch M_SAP: 2 counters, then one flag per domain (zero at rest)
-  bool force_generic_sap = false;  // testing: use the generic SAP kernel
   int sap_shape = -1;              // SAP block-kernel shape: -1 autotuned, else an index of the shapes
   bool sap_general = false;        // SAP on domains sap_dom, independent of the storage blocking
   int sap_dom[4] = {0, 0, 0, 0};
@@ -805,10 +804,16 @@ void sap_staged_sequence_f16(qcd_ctx* ctx, F32Spinor s_first_in, F16Spinor s, F3
                              float4* halo, int nrhs, int n_sap, int n_jac, cudaStream_t st);
 void sap_staged_sequence_h16g(qcd_ctx* ctx, F32Spinor s_first_in, F32Spinor s, F32Spinor x, F32Spinor b,
                               float4* halo, int nrhs, int n_sap, int n_jac, cudaStream_t st);
-// ws_x16 holds 96 bytes per site and right-hand side: the float16 x of the
-// generic kernel, or the face halo of the shared-memory kernel
+// the same half-sweeps with four threads per site, any storage block (sap_split.cu)
+void sap_split_f32(qcd_ctx* ctx, F32Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
+                   cudaStream_t st);
+void sap_split_f16(qcd_ctx* ctx, F16Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
+                   cudaStream_t st);
+void sap_split_h16g(qcd_ctx* ctx, F32Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
+                    cudaStream_t st);
+// halo: 96 bytes per site and right-hand side
 void sap_apply_launch(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n_sap, int n_jac, int sap_prec,
-                      void* ws_s, void* ws_x16, void* ws_b16, cudaStream_t st);
+                      void* ws_s, void* halo, cudaStream_t st);
 void workspace_reset_graphs(qcd_ctx* ctx);
 // SAP on the context's general domains (sap_dom, any extents; up to 1152
 // sites on the one-CTA kernel, larger ones on the cluster kernel)

@@ -1081,16 +1081,28 @@ static void flow_sequence(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, SIO x, F3
 // its staged operator.  qcd_set_sap_shape fixes the shape.
 // The last two shapes run the whole of M_SAP in one launch (sap_flow_kernel),
 // the second of them with half of its CTAs starting later, so that the
-// CTAs on one SM load their operators at different times.
+// CTAs on one SM load their operators at different times.  While a colour's
+// domains and right-hand sides fit one wave of the block kernel
+// (kSplitItems), the tuner also tries the kernel with four threads per site
+// (sap_split.cu), which wins up to about 16 domains a colour.
 static const char* const kSapShapes[] = {"256x1site", "128x2sites", "256x1site_rhs_grid", "one_launch",
-                                         "one_launch_staggered"};
+                                         "one_launch_staggered", "4threads_per_site"};
+constexpr int kSplitShape = 5;
+constexpr long long kSplitItems = 304;
 constexpr int kFlowStaggerNs = 10000;
 
 template <bool HALF, typename SIO>
 static void staged_sequence(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, SIO x, F32Spinor b, F32Spinor x_out32,
                             float4* halo, int nrhs, int n_sap, int n_jac, cudaStream_t st) {
   auto run = [&](int v) {
-    if (v == 1)
+    if (v == kSplitShape) {
+      if constexpr (std::is_same<SIO, F16Spinor>::value)
+        sap_split_f16(ctx, s, x_out32, b, nrhs, n_sap, n_jac, st);
+      else if constexpr (HALF)
+        sap_split_h16g(ctx, s, x, b, nrhs, n_sap, n_jac, st);
+      else
+        sap_split_f32(ctx, s, x, b, nrhs, n_sap, n_jac, st);
+    } else if (v == 1)
       staged_sequence_shape<HALF, SIO, 2>(ctx, s_first_in32, s, x, b, x_out32, halo, nrhs, n_sap, n_jac, st);
     else if (v >= 3 && n_sap >= 1)
       flow_sequence<HALF, SIO>(ctx, s_first_in32, s, x, b, x_out32, halo, nrhs, n_sap, n_jac, st,
@@ -1108,12 +1120,23 @@ static void staged_sequence(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, SIO x, 
                   g.L[3], nrhs, n_sap, n_jac);
     // candidates: both thread shapes, the right-hand-side grid (several
     // right-hand sides only) and, with n_sap >= 1, the two one-launch forms
-    static const int with_rhs[] = {0, 1, 2, 3, 4}, one_rhs[] = {0, 1, 3, 4};
-    const int* cand = nrhs > 1 ? with_rhs : one_rhs;
-    const int nc = (nrhs > 1 ? 3 : 2) + (n_sap >= 1 ? 2 : 0);
-    const char* names[5];
-    for (int c = 0; c < nc; ++c) names[c] = kSapShapes[cand[c]];
+    int cand[6], nc = 0;
+    const char* names[6];
+    auto add = [&](int c) {
+      names[nc] = kSapShapes[c];
+      cand[nc++] = c;
+    };
+    add(0);
+    add(1);
+    if (nrhs > 1) add(2);
+    if (n_sap >= 1) {
+      add(3);
+      add(4);
+    }
+    if ((long long)g.nhalf * nrhs <= kSplitItems) add(kSplitShape);
     v = cand[tune_pick(ctx, key, nc, names, [&](int c) { run(cand[c]); }, st)];
+    // a failure hook concerns the block kernel's waits, which the split one does not have
+    if (v == kSplitShape && ctx->inject != QCD_INJECT_NONE) v = 0;
   }
   run(v);
 }

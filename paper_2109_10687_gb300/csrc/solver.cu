@@ -34,7 +34,7 @@ struct Workspace {
   size_t v4 = 0;  // float4 per rhs
   float4 *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *t = nullptr, *zp = nullptr, *zr = nullptr,
          *rt = nullptr, *tmp32 = nullptr;
-  void *sap_s = nullptr, *sap_x16 = nullptr, *sap_b16 = nullptr;
+  void *sap_s = nullptr, *sap_halo = nullptr;
   double2 *x64 = nullptr, *r64 = nullptr, *b64 = nullptr, *t64 = nullptr;
   double* partials = nullptr;
   double* dres = nullptr;   // small device results: 4 doubles per rhs
@@ -75,7 +75,7 @@ void workspace_reset_graphs(qcd_ctx* ctx) {
 void workspace_free(qcd_ctx* ctx) {
   Workspace* w = ctx->ws;
   if (!w) return;
-  void* ptrs[] = {w->x, w->r, w->p, w->q, w->t, w->zp, w->zr, w->rt, w->tmp32, w->sap_s, w->sap_x16, w->sap_b16,
+  void* ptrs[] = {w->x, w->r, w->p, w->q, w->t, w->zp, w->zr, w->rt, w->tmp32, w->sap_s, w->sap_halo,
                   w->x64, w->r64, w->b64, w->t64, w->partials, w->dres, w->counters, w->scal};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -128,9 +128,8 @@ static Workspace* workspace(qcd_ctx* ctx, int nrhs, bool solver) {
     double2** v64[] = {&w->x64, &w->r64, &w->b64, &w->t64};
     for (auto v : v64) QCD_CUDA_CHECK(cudaMalloc(v, b64));
     QCD_CUDA_CHECK(cudaMalloc(&w->sap_s, spinor_bytes(g, QCD_PREC_SINGLE) * keep_nrhs));
-    // float16 x of the generic SAP kernel, or the shared-memory kernel's halo (96 B per site)
-    QCD_CUDA_CHECK(cudaMalloc(&w->sap_x16, spinor_bytes(g, QCD_PREC_SINGLE) * keep_nrhs));
-    QCD_CUDA_CHECK(cudaMalloc(&w->sap_b16, spinor_bytes(g, QCD_PREC_HALF) * keep_nrhs));
+    // face halo of the SAP block kernel, 96 B per site
+    QCD_CUDA_CHECK(cudaMalloc(&w->sap_halo, spinor_bytes(g, QCD_PREC_SINGLE) * keep_nrhs));
   }
   return w;
 }
@@ -619,7 +618,7 @@ struct Launcher {
 
 static void am_sap(qcd_ctx* ctx, Workspace* w, float4* z, float4* out, const float4* in, int nrhs, int n_sap, int n_jac,
                    int sap_prec, cudaStream_t st) {
-  sap_apply_launch(ctx, z, in, nrhs, n_sap, n_jac, sap_prec, w->sap_s, w->sap_x16, w->sap_b16, st);
+  sap_apply_launch(ctx, z, in, nrhs, n_sap, n_jac, sap_prec, w->sap_s, w->sap_halo, st);
   dslash_launch(ctx, out, z, QCD_PREC_SINGLE, MODE_A, nrhs, st);
 }
 
@@ -689,7 +688,7 @@ static int bicgstab_sap(qcd_ctx* ctx, Workspace* w, const float4* b32, int nrhs,
     // operator and SAP kernels of the loop once beforehand (into scratch
     // buffers the loop overwrites before reading; p holds the source here)
     dslash_launch(ctx, w->t, w->zp, QCD_PREC_SINGLE, MODE_A, nrhs, st);
-    sap_apply_launch(ctx, w->zr, w->p, nrhs, P.n_sap, P.n_jac, P.sap_prec, w->sap_s, w->sap_x16, w->sap_b16, st);
+    sap_apply_launch(ctx, w->zr, w->p, nrhs, P.n_sap, P.n_jac, P.sap_prec, w->sap_s, w->sap_halo, st);
     cudaGraph_t gr;
     const long long c_start = ctx->launches;
     long long c0 = c_start;
@@ -879,8 +878,8 @@ extern "C" int qcd_sap_apply_nrhs(qcd_ctx* ctx, void* out, const void* in, int n
   if (with_A) {
     am_sap(ctx, w, w->tmp32, (float4*)out, (const float4*)in, nrhs, n_sap, n_jac, sap_prec, st);
   } else {
-    sap_apply_launch(ctx, (float4*)out, (const float4*)in, nrhs, n_sap, n_jac, sap_prec, w->sap_s, w->sap_x16,
-                     w->sap_b16, st);
+    sap_apply_launch(ctx, (float4*)out, (const float4*)in, nrhs, n_sap, n_jac, sap_prec, w->sap_s, w->sap_halo,
+                     st);
   }
   API_END(ctx)
 }
