@@ -926,6 +926,23 @@ constexpr int st_smem_bytes() {
   return SX_BYTES + StageT<HALF>::LINK_BYTES + StageT<HALF>::CLOV_BYTES + 32;
 }
 
+// More than half of an SM's shared memory.  A launch of no more blocks than
+// SMs asks for this much, so that each block gets an SM of its own: with room
+// for two, and the next launch's blocks arriving while this one's still run,
+// they pair up on some SMs and leave others idle (float16 M_SAP at 16^4, 128
+// blocks a launch: 0.229 -> 0.142 ms).
+constexpr int ST_ONE_PER_SM = 120 * 1024;
+template <bool HALF>
+static int st_launch_smem(long long blocks) {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    QCD_CUDA_CHECK(cudaGetDevice(&dev));
+    QCD_CUDA_CHECK(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n;
+  }();
+  return HALF && blocks <= sms ? ST_ONE_PER_SM : st_smem_bytes<HALF>();
+}
+
 void sap_staging_alloc(qcd_ctx* ctx) {
   const Geom& g = ctx->geom;
   if (!(g.d[0] == 4 && g.d[1] == 4 && g.d[2] == 4 && g.d[3] == 4)) return;
@@ -938,13 +955,13 @@ void sap_staging_alloc(qcd_ctx* ctx) {
     const int s16 = st_smem_bytes<true>();
     const int s32 = st_smem_bytes<false>();
     QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_staged_kernel<true, F16Spinor, 1>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, s16));
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, ST_ONE_PER_SM));
     QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_staged_kernel<true, F16Spinor, 2>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, s16));
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, ST_ONE_PER_SM));
     QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_staged_kernel<true, F32Spinor, 1>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, s16));
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, ST_ONE_PER_SM));
     QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_staged_kernel<true, F32Spinor, 2>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, s16));
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, ST_ONE_PER_SM));
     QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_staged_kernel<false, F32Spinor, 1>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, s32));
     QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_staged_kernel<false, F32Spinor, 2>,
@@ -1008,7 +1025,7 @@ static void staged_sequence_shape(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, S
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(ctx->geom.nhalf, rhs_grid ? nrhs : 1);
       cfg.blockDim = dim3(ST_THREADS / SPT);
-      cfg.dynamicSmemBytes = st_smem_bytes<HALF>();
+      cfg.dynamicSmemBytes = st_launch_smem<HALF>((long long)cfg.gridDim.x * cfg.gridDim.y);
       cfg.stream = st;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
