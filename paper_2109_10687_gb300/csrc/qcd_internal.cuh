@@ -804,7 +804,14 @@ void sap_staged_sequence_f16(qcd_ctx* ctx, F32Spinor s_first_in, F16Spinor s, F3
                              float4* halo, int nrhs, int n_sap, int n_jac, cudaStream_t st);
 void sap_staged_sequence_h16g(qcd_ctx* ctx, F32Spinor s_first_in, F32Spinor s, F32Spinor x, F32Spinor b,
                               float4* halo, int nrhs, int n_sap, int n_jac, cudaStream_t st);
-// the same half-sweeps with four threads per site, any storage block (sap_split.cu)
+// the same half-sweeps on any storage block, a thread per site (sap_block.cu) ...
+void sap_block_f32(qcd_ctx* ctx, F32Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
+                   cudaStream_t st);
+void sap_block_f16(qcd_ctx* ctx, F16Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
+                   cudaStream_t st);
+void sap_block_h16g(qcd_ctx* ctx, F32Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
+                    cudaStream_t st);
+// ... and with four threads per site (sap_split.cu)
 void sap_split_f32(qcd_ctx* ctx, F32Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
                    cudaStream_t st);
 void sap_split_f16(qcd_ctx* ctx, F16Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,

@@ -26,7 +26,7 @@ namespace qcd {
 // sized for nrhs right-hand sides, which go through every launch together.
 // Domains set apart from the storage blocks have kernels of their own; 4^4
 // storage blocks take the block kernel (which on small lattices may hand over
-// to the split one), all others the split kernel.
+// to the split one), all others the kernel of sap_block.cu.
 void sap_apply_launch(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n_sap, int n_jac, int sap_prec,
                       void* ws_s, void* halo, cudaStream_t st) {
   if (ctx->sap_general) {
@@ -40,13 +40,13 @@ void sap_apply_launch(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n_
   float4* h = (float4*)halo;
   if (sap_prec == QCD_PREC_HALF) {  // float16 links, C_inv and s
     if (staged) sap_staged_sequence_f16(ctx, bs, s16, bs, xs, h, nrhs, n_sap, n_jac, st);
-    else sap_split_f16(ctx, s16, xs, bs, nrhs, n_sap, n_jac, st);
+    else sap_block_f16(ctx, s16, xs, bs, nrhs, n_sap, n_jac, st);
   } else if (sap_prec == QCD_PREC_HALF_GAUGE) {  // float16 links and C_inv, float32 vectors
     if (staged) sap_staged_sequence_h16g(ctx, bs, s32, xs, bs, h, nrhs, n_sap, n_jac, st);
-    else sap_split_h16g(ctx, s32, xs, bs, nrhs, n_sap, n_jac, st);
+    else sap_block_h16g(ctx, s32, xs, bs, nrhs, n_sap, n_jac, st);
   } else {
     if (staged) sap_staged_sequence_f32(ctx, bs, s32, xs, bs, h, nrhs, n_sap, n_jac, st);
-    else sap_split_f32(ctx, s32, xs, bs, nrhs, n_sap, n_jac, st);
+    else sap_block_f32(ctx, s32, xs, bs, nrhs, n_sap, n_jac, st);
   }
 }
 

@@ -1,6 +1,6 @@
-// SAP half-sweep with four threads per site (Sec. 3 of arXiv:2109.10687,
-// Algorithms 1 and 2): every storage-block domain that is not 4^4, and 4^4
-// domains on lattices with too few of them to fill the GPU.
+// SAP half-sweep on 4^4 domains with four threads per site (Sec. 3 of
+// arXiv:2109.10687, Algorithms 1 and 2), for lattices with too few domains to
+// fill the GPU.
 //
 // Per launch, for the domains of one colour c: the surface term
 // s <- s + kappa C_inv H_cc' x_c', n_jac Jacobi sweeps
@@ -10,8 +10,8 @@
 //
 // What bounds it: a small lattice leaves a thread per site with two warps per
 // scheduler, each waiting on its own chain of loads and multiply-adds.  So a
-// site gets four threads and a block 64 sites, and a domain of more than 64
-// sites a thread-block cluster (one block per 64).
+// site gets four threads, a block 64 sites (a time slice of the domain) and a
+// domain a cluster of four blocks.
 //   Hops: thread (site, direction) keeps U_mu(n) and U_mu(n - mu) in
 //     registers for the whole launch, already converted to float32, reads the
 //     two neighbours' spinors (the neighbouring block's through distributed
@@ -27,9 +27,8 @@
 // M_SAP (n_sap 4, n_jac 4): 8^4 on 4^4 domains, float32, 0.134 ms with a thread
 // per site (8 blocks a colour) and 0.105 ms here (32 blocks); 16 8^3 0.134 and
 // 0.121; from 16^2 8^2 on (32 domains a colour) the block kernel is the faster.
-// 12x20x12x28 on 2^4 domains, float32, 0.48 ms with a thread per site reading
-// links and C_inv through L1 and 0.40 ms here.  It is bound by shared memory
-// (2.2 KB per site and sweep) in turn with the FMA pipe, between barriers.
+// It is bound by shared memory (2.2 KB per site and sweep) in turn with the FMA
+// pipe, between barriers.
 
 #include <cooperative_groups.h>
 
@@ -44,6 +43,7 @@ namespace qcd {
 
 constexpr int SP_SITES = 64;
 constexpr int SP_THREADS = 4 * SP_SITES;
+constexpr int SP_BLOCKS = 4;                 // blocks per domain (cluster size)
 constexpr int SP_XF4 = 6 * SP_SITES;         // float4 of one buffer of x
 constexpr int SP_HF2 = 8 * 6 * SP_SITES;     // float2 of the half spinors [hop 8][row 2][colour 3][site]
 
@@ -226,9 +226,9 @@ __device__ __forceinline__ float2* sp_comp(const F32Spinor& f, const Geom& g, in
   return reinterpret_cast<float2*>(f.p + f.idx(g, dom, comp >> 1, s)) + (comp & 1);
 }
 
-template <bool HALF, typename SIO, bool CLUSTER>
+template <bool HALF, typename SIO>
 __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF, SIO> a) {
-  __shared__ float4 xs[(CLUSTER ? 2 : 1) * SP_XF4];
+  __shared__ float4 xs[2 * SP_XF4];
   __shared__ float2 hs[SP_HF2];
   __shared__ float2 ex[4 * 3 * SP_SITES];
   __shared__ float4 zero4;
@@ -240,12 +240,9 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // direction in the hops, spin in the site sums
   const int q = w >> 1, site = (w & 1) * 32 + lane;
-  // a block's 64 sites are consecutive sites of the colour's domains; sites
-  // past the last repeat the first and store nothing
-  const int total = g.nhalf << g.logvd, first = blockIdx.x * SP_SITES;
-  const bool live = first + site < total;
-  const int k0 = live ? first + site : first;
-  const int dom = a.colour * g.nhalf + (k0 >> g.logvd), loc = k0 & (g.vd - 1);
+  const cg::cluster_group cl = cg::this_cluster();
+  const int dom = a.colour * g.nhalf + blockIdx.x / SP_BLOCKS;
+  const int loc = (int)cl.block_rank() * SP_SITES + site;  // site of the domain
   const int rhs_off = blockIdx.y * g.ndom;
   const int domr = dom + rhs_off;
 
@@ -257,15 +254,8 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
   sp_link<HALF>(a.links, g, bd, q, bs, ub);
   const bool fin = hop_is_intra(g, loc, q, true), bin = hop_is_intra(g, loc, q, false);
   const float4 *pf = &zero4, *pb = &zero4;
-  if (CLUSTER) {
-    // a domain is a cluster: block (site >> 6), position site & 63
-    cg::cluster_group cl = cg::this_cluster();
-    if (fin) pf = cl.map_shared_rank(xs, fs / SP_SITES) + fs % SP_SITES;
-    if (bin) pb = cl.map_shared_rank(xs, bs / SP_SITES) + bs % SP_SITES;
-  } else {
-    if (fin) pf = xs + site + (fs - loc);
-    if (bin) pb = xs + site + (bs - loc);
-  }
+  if (fin) pf = cl.map_shared_rank(xs, fs / SP_SITES) + fs % SP_SITES;
+  if (bin) pb = cl.map_shared_rank(xs, bs / SP_SITES) + bs % SP_SITES;
   const int sf = fin ? SP_SITES : 0, sb = bin ? SP_SITES : 0;
   CinvRows m;
   sp_switch(q, [&](auto k) { sp_cinv<HALF, decltype(k)::value>(a.cinv, g, dom, loc, m); });
@@ -300,11 +290,6 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
       reinterpret_cast<float2*>(p + (k >> 1) * SP_SITES)[k & 1] = make_float2(v[c].re, v[c].im);
     }
   };
-  auto sync_all = [&]() {
-    if (CLUSTER) cg::this_cluster().sync();
-    else __syncthreads();
-  };
-
   if (a.do_surface) {
     sp_switch(q, [&](auto k) {
       constexpr int MU = decltype(k)::value;
@@ -322,7 +307,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
     for (int c = 0; c < 3; ++c) src[c] = cfma(a.kappa, y[c], src[c]);
   }
   put_x(src, 0);
-  sync_all();
+  cl.sync();
 
   cx<float> xk[3] = {src[0], src[1], src[2]};
   const int napp = a.n_jac + (a.do_update ? 1 : 0);
@@ -330,7 +315,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
   for (int it = 0; it < napp; ++it) {
     sp_switch(q, [&](auto k) {
       constexpr int MU = decltype(k)::value;
-      const int off = CLUSTER ? cur * SP_XF4 : 0;
+      const int off = cur * SP_XF4;
       Spinor<float> p;
       sp_read(pf + (fin ? off : 0), sf, p);
       sp_hop_fwd<MU>(uf, p, 1.f, hs, site);
@@ -342,9 +327,9 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
     if (it < a.n_jac) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) xk[c] = cfma(a.kappa, y[c], src[c]);
-      if (CLUSTER) cur ^= 1;  // the other blocks may still read this one's x
+      cur ^= 1;  // the other blocks may still read this one's x
       put_x(xk, cur);
-      sync_all();
+      cl.sync();
     } else {
       cx<float> v[3];
       float mx = 0.f;
@@ -355,31 +340,27 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
         mx = fmaxf(mx, fmaxf(fabsf(v[c].re), fabsf(v[c].im)));
       }
       if constexpr (std::is_same<SIO, F32Spinor>::value) {
-        if (live)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) *sp_comp(a.s_out, g, domr, 3 * q + c, loc) = make_float2(v[c].re, v[c].im);
+        for (int c = 0; c < 3; ++c) *sp_comp(a.s_out, g, domr, 3 * q + c, loc) = make_float2(v[c].re, v[c].im);
       } else {
         // the site's norm is the largest component of all four spins
         nrm[q * SP_SITES + site] = mx;
         __syncthreads();
         mx = fmaxf(fmaxf(nrm[site], nrm[SP_SITES + site]), fmaxf(nrm[2 * SP_SITES + site], nrm[3 * SP_SITES + site]));
         const float inv = mx > 0.f ? 1.0f / mx : 0.f;
-        if (live) {
-          if (q == 0) a.s_out.nrm[((size_t)domr << g.logvd) + loc] = mx;
+        if (q == 0) a.s_out.nrm[((size_t)domr << g.logvd) + loc] = mx;
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const int k = 3 * q + c;
-            const __half2 h = __floats2half2_rn(v[c].re * inv, v[c].im * inv);
-            reinterpret_cast<__half2*>(a.s_out.p + a.s_out.idx(g, domr, k >> 2, loc))[k & 3] = h;
-          }
+        for (int c = 0; c < 3; ++c) {
+          const int k = 3 * q + c;
+          const __half2 h = __floats2half2_rn(v[c].re * inv, v[c].im * inv);
+          reinterpret_cast<__half2*>(a.s_out.p + a.s_out.idx(g, domr, k >> 2, loc))[k & 3] = h;
         }
       }
     }
   }
-  if (live)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) *sp_comp(a.x, g, domr, 3 * q + c, loc) = make_float2(xk[c].re, xk[c].im);
-  if (CLUSTER) cg::this_cluster().sync();  // the neighbours' last reads of this block's x are done
+  for (int c = 0; c < 3; ++c) *sp_comp(a.x, g, domr, 3 * q + c, loc) = make_float2(xk[c].re, xk[c].im);
+  cl.sync();  // the neighbours' last reads of this block's x are done
 }
 
 // Algorithm 1 as 2 (n_sap + 1) launches, every right-hand side in each.
@@ -399,9 +380,6 @@ static void split_sequence(qcd_ctx* ctx, SIO s, F32Spinor x, F32Spinor b, int nr
   a.b = b;
   a.links = HALF ? (const void*)ctx->u16 : (const void*)ctx->u32;
   a.cinv = HALF ? (const void*)ctx->cinv16 : (const void*)ctx->cinv32;
-  const long long sites = (long long)g.nhalf << g.logvd;
-  QCD_REQUIRE(sites + SP_SITES < (1LL << 31), QCD_ERR_ARG, "SAP: lattice too large");
-  const bool cluster = g.vd > SP_SITES;
   for (int sweep = 0; sweep <= n_sap; ++sweep) {
     a.s_in32 = sweep == 0 ? b : F32Spinor{nullptr};
     a.do_update = sweep == n_sap ? 0 : 1;
@@ -410,20 +388,19 @@ static void split_sequence(qcd_ctx* ctx, SIO s, F32Spinor x, F32Spinor b, int nr
       a.do_surface = (sweep == 0 && colour == 0) ? 0 : 1;
       LaunchScope ls(ctx, QCD_KC_SAP_BLOCK, st);
       cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)((sites + SP_SITES - 1) / SP_SITES), nrhs);
+      cfg.gridDim = dim3(g.nhalf * SP_BLOCKS, nrhs);
       cfg.blockDim = dim3(SP_THREADS);
       cfg.stream = st;
       cudaLaunchAttribute attr[2];
       attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
       attr[0].val.programmaticStreamSerializationAllowed = 1;
       attr[1].id = cudaLaunchAttributeClusterDimension;
-      attr[1].val.clusterDim.x = cluster ? g.vd / SP_SITES : 1;
+      attr[1].val.clusterDim.x = SP_BLOCKS;
       attr[1].val.clusterDim.y = 1;
       attr[1].val.clusterDim.z = 1;
       cfg.attrs = attr;
-      cfg.numAttrs = cluster ? 2 : 1;
-      if (cluster) QCD_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sap_split_kernel<HALF, SIO, true>, a));
-      else QCD_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sap_split_kernel<HALF, SIO, false>, a));
+      cfg.numAttrs = 2;
+      QCD_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sap_split_kernel<HALF, SIO>, a));
       check_launch();
     }
   }

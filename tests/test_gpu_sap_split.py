@@ -1,8 +1,9 @@
-"""The SAP kernel with four threads per site against the oracle and, on 4^4
-domains, against the block kernel bit for bit: domains smaller than a block of
-64 sites, of exactly one block and of a cluster of two and four; a last block
-that is not full; hops of width-one domains that all leave; one and three
-right-hand sides."""
+"""The SAP kernel of storage blocks other than 4^4 against the oracle: domains
+of less than, exactly and more than a block of 64 sites; a last block that is
+not full; directions in which a domain is one site wide (every hop leaves), two
+(one body for both hops) and more; one and three right-hand sides.  And the
+kernel with four threads per site against the block kernel of 4^4 domains, bit
+for bit."""
 
 import numpy as np
 import pytest
