@@ -7,16 +7,29 @@
 // site.  At entry a CTA brings its slice's links (float16, 40 B per link)
 // and C_inv (float16, 144 B per site) into shared memory with two bulk
 // copies on an mbarrier (bounded wait), from a staging layout built for this
-// kernel.  Its shared memory also holds two buffers of the slice's float32
-// iterate x.  A Jacobi sweep reads x from the current buffer and writes the
-// other: hops in x, y and z stay inside the slice; the t hops read the
-// neighbouring slice's x, and for a backward hop its link, from that CTA's
-// shared memory through the cluster's distributed shared memory.  One
-// cluster barrier per sweep separates the reads of a buffer from the next
-// writes to it.  The surface term (hops that leave the domain) reads the
-// other colour's x and the neighbouring domains' links from memory.
-// Before a CTA leaves, a last cluster barrier keeps its shared memory alive
-// while its neighbours may still read it.
+// kernel.  Its shared memory also holds the slice's float32 iterate x and, for the hops in t, two half
+// spinors per site that the neighbouring slices' CTAs write there through
+// distributed shared memory: P- x(t + 1) from above and U^dag P+ x(t - 1),
+// finished by the CTA that holds the link, from below.  Hops in x, y and z
+// read x of the own slice, without branches: a hop that leaves the domain
+// reads a site of zeros.
+//
+// Two cluster barriers per sweep: the first (arrive after the hops' reads,
+// wait after the C_inv multiply) separates the reads of x and of the half
+// spinors from the next writes, the second those writes from the next reads.
+//
+// The surface term (hops that leave the domain) reads the other colour's x
+// and the neighbouring domains' links from memory; its lines are prefetched
+// to L1 while the staging copies are under way.  (One CTA fills an SM, so an
+// early start of the next launch would gain nothing; without it L1 holds no
+// line of an earlier launch.)
+//
+// What bounds it: one CTA of 12 warps per SM (16x6x4x3: 190 KB of shared
+// memory), so each warp's chain of loads and multiply-adds.  Reading the
+// t neighbours' spinors and links from the other CTAs in place, with a branch
+// per hop, a sweep took 6.7 us for the clusters resident at a time and the rest
+// of a launch 13 us; now 3.8 and 12.7 us (32x24x16x24, 128 clusters in three
+// waves: a half-sweep with n_jac 2 96 -> 70 us).
 
 #include <cooperative_groups.h>
 
@@ -32,7 +45,9 @@ constexpr int CS_MAX_K = 8;            // slices (CTAs) per cluster, the portabl
 constexpr int CS_MAX_SLICE = 448;      // sites per slice: 496 B of shared memory each
 constexpr int CS_LINK_H2 = 10;         // half2 per staged link (9 + 1 pad)
 constexpr int CS_CLOV_U4 = 9;          // uint4 per site of staged C_inv
-constexpr int CS_BYTES_PER_SITE = 2 * 96 + 4 * CS_LINK_H2 * 4 + CS_CLOV_U4 * 16;  // 496
+constexpr int CS_BYTES_PER_SITE = 96 + 2 * 48 + 4 * CS_LINK_H2 * 4 + CS_CLOV_U4 * 16;  // 496
+constexpr int CS_GHOST = 8;            // zero sites after x, one per 16-byte bank group
+constexpr int CS_EXTRA_BYTES = 6 * CS_GHOST * 16 + 16;
 
 struct ClusterSapArgs {
   Geom g;
@@ -96,18 +111,35 @@ __device__ __forceinline__ void cs_clover(const unsigned char* base, int site, S
   }
 }
 
-__device__ __forceinline__ void cs_load_x(const float4* buf, int slice, int s, Spinor<float>& a) {
+// x: float4 [6][slice + CS_GHOST]
+__device__ __forceinline__ void cs_load_x(const float4* buf, int stride, int s, Spinor<float>& a) {
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    const float4 v = buf[k * slice + s];
+    const float4 v = buf[k * stride + s];
     a.v[(2 * k) / 3][(2 * k) % 3] = make_cx(v.x, v.y);
     a.v[(2 * k + 1) / 3][(2 * k + 1) % 3] = make_cx(v.z, v.w);
   }
 }
-__device__ __forceinline__ void cs_store_x(float4* buf, int slice, int s, const Spinor<float>& a) {
+__device__ __forceinline__ void cs_store_x(float4* buf, int stride, int s, const Spinor<float>& a) {
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const cx<float> a0 = a.v[(2 * k) / 3][(2 * k) % 3], a1 = a.v[(2 * k + 1) / 3][(2 * k + 1) % 3];
+    buf[k * stride + s] = make_float4(a0.re, a0.im, a1.re, a1.im);
+  }
+}
+// half spinors: float4 [3][slice]
+__device__ __forceinline__ void cs_load_half(const float4* buf, int slice, int s, HalfSpinor<float>& h) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float4 v = buf[k * slice + s];
+    h.h[(2 * k) / 3][(2 * k) % 3] = make_cx(v.x, v.y);
+    h.h[(2 * k + 1) / 3][(2 * k + 1) % 3] = make_cx(v.z, v.w);
+  }
+}
+__device__ __forceinline__ void cs_store_half(float4* buf, int slice, int s, const HalfSpinor<float>& h) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const cx<float> a0 = h.h[(2 * k) / 3][(2 * k) % 3], a1 = h.h[(2 * k + 1) / 3][(2 * k + 1) % 3];
     buf[k * slice + s] = make_float4(a0.re, a0.im, a1.re, a1.im);
   }
 }
@@ -121,20 +153,64 @@ __device__ __forceinline__ void cs_hop(const SU3<float>& u, const Spinor<float>&
   accumulate<MU, PM>(acc, uh, sign);
 }
 
-// hops of direction MU (0..2) that stay in the slice
+// both hops of direction MU (0..2): the neighbours' sites in the slice, or a
+// zero site (and some valid link) for a hop that leaves the domain
 template <int MU>
-__device__ __forceinline__ void cs_intra_space(const ClusterSapArgs& a, const float4* xb, const unsigned char* sl,
-                                               const int lc[4], int s, Spinor<float>& acc) {
-  const int stride = MU == 0 ? 1 : (MU == 1 ? a.sd[0] : a.sd[0] * a.sd[1]);
-  if (lc[MU] < a.sd[MU] - 1) {
-    Spinor<float> p;
-    cs_load_x(xb, a.slice, s + stride, p);
-    cs_hop<MU, -1>(cs_link(sl, a.slice, MU, s), p, 1.f, acc);
+__device__ __forceinline__ void cs_intra_space(const float4* xb, const unsigned char* sl, int slice, int s, int stride,
+                                               bool fin, bool bin, Spinor<float>& acc) {
+  const int zero_site = slice + (s & (CS_GHOST - 1));
+  Spinor<float> p;
+  cs_load_x(xb, slice + CS_GHOST, fin ? s + stride : zero_site, p);
+  cs_hop<MU, -1>(cs_link(sl, slice, MU, s), p, 1.f, acc);
+  cs_load_x(xb, slice + CS_GHOST, bin ? s - stride : zero_site, p);
+  cs_hop<MU, +1>(cs_link(sl, slice, MU, bin ? s - stride : s), p, 1.f, acc);
+}
+
+// this site's half spinors for the neighbouring slices' t hops, into their
+// CTAs' shared memory (null: no such slice)
+__device__ __forceinline__ void cs_push_t(float4* below, float4* above, const unsigned char* sl, int slice, int s,
+                                          const Spinor<float>& x) {
+  HalfSpinor<float> h, uh;
+  if (below) {
+    project<3, -1>(x, h);
+    cs_store_half(below, slice, s, h);
   }
-  if (lc[MU] > 0) {
-    Spinor<float> p;
-    cs_load_x(xb, a.slice, s - stride, p);
-    cs_hop<MU, +1>(cs_link(sl, a.slice, MU, s - stride), p, 1.f, acc);
+  if (above) {
+    project<3, +1>(x, h);
+    su3_dag_mul(cs_link(sl, slice, 3, s), h, uh);
+    cs_store_half(above, slice, s, uh);
+  }
+}
+
+__device__ __forceinline__ void cs_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cs_wait_all() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// L1 prefetch of what cs_inter reads for one hop: the spinor and, for a
+// backward hop, the neighbouring domain's link
+__device__ __forceinline__ void cs_prefetch(const ClusterSapArgs& a, const int Y[4], int mu, bool bwd) {
+  const Geom& g = a.g;
+  int nd, ns;
+  coords_to_internal(g, Y, nd, ns);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.x.p + a.x.idx(g, nd, k, ns)));
+  if (bwd) {
+    const __half2* p = a.U16.p + (((size_t)((nd * 4 + mu) * 9)) << g.logvd) + ns;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) asm volatile("prefetch.global.L1 [%0];" ::"l"(p + ((size_t)e << g.logvd)));
+  }
+}
+__device__ __forceinline__ void cs_prefetch_surface(const ClusterSapArgs& a, const int X[4], const int lc[4]) {
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    int Y[4] = {X[0], X[1], X[2], X[3]};
+    if (lc[mu] == a.sd[mu] - 1) {
+      Y[mu] = X[mu] + 1 == a.g.L[mu] ? 0 : X[mu] + 1;
+      cs_prefetch(a, Y, mu, false);
+    }
+    if (lc[mu] == 0) {
+      Y[mu] = X[mu] == 0 ? a.g.L[mu] - 1 : X[mu] - 1;
+      cs_prefetch(a, Y, mu, true);
+    }
   }
 }
 
@@ -196,9 +272,10 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
   const int K = a.sd[3];
   const int lt = (int)cl.block_rank();  // time slice of this CTA
   const int S = a.slice;
-  float4* xbuf0 = reinterpret_cast<float4*>(csm);
-  float4* xbuf1 = xbuf0 + 6 * S;
-  unsigned char* sl = csm + 2 * 96 * S;          // links
+  float4* xb = reinterpret_cast<float4*>(csm);   // the iterate
+  float4* t_up = xb + 6 * (S + CS_GHOST);        // P- x of the slice above
+  float4* t_dn = t_up + 3 * S;                   // U^dag P+ x of the slice below
+  unsigned char* sl = reinterpret_cast<unsigned char*>(t_dn + 3 * S);  // links
   unsigned char* sc = sl + 4 * CS_LINK_H2 * 4 * S;  // C_inv
   uint64_t* bar = reinterpret_cast<uint64_t*>(sc + CS_CLOV_U4 * 16 * S);
   int* bad = reinterpret_cast<int*>(bar + 1);
@@ -245,8 +322,13 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
   for (int mu = 0; mu < 4; ++mu) X[mu] = D[mu] * a.sd[mu] + lc[mu];
   int dom, st;
   coords_to_internal(g, X, dom, st);
+  for (int i = tid; i < 6 * CS_GHOST; i += blockDim.x)
+    xb[(i / CS_GHOST) * (S + CS_GHOST) + S + i % CS_GHOST] = make_float4(0.f, 0.f, 0.f, 0.f);
   Spinor<float> src;
-  if (live) a.s_in.load(g, dom, st, src);
+  if (live) {
+    if (a.do_surface) cs_prefetch_surface(a, X, lc);
+    a.s_in.load(g, dom, st, src);
+  }
   __syncthreads();  // barrier initialisation visible to every thread
   {
     // every CTA of the cluster takes the same decision on a wait that gave up
@@ -279,34 +361,38 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
         src.v[sp][c].im = fmaf(a.kappa, acc.v[sp][c].im, src.v[sp][c].im);
       }
   }
-  if (live) cs_store_x(xbuf0, S, s, src);
-  cl.sync();  // every slice holds x_0
-  int cur = 0;
+  float4* below = lt > 0 ? cl.map_shared_rank(t_up, lt - 1) : nullptr;
+  float4* above = lt < K - 1 ? cl.map_shared_rank(t_dn, lt + 1) : nullptr;
+  if (live) {
+    cs_store_x(xb, S + CS_GHOST, s, src);
+    cs_push_t(below, above, sl, S, s, src);
+  }
+  cs_arrive();
+  cs_wait_all();  // every slice holds x_0 and its neighbours' half spinors
+  const bool fx = lc[0] < a.sd[0] - 1, fy = lc[1] < a.sd[1] - 1, fz = lc[2] < a.sd[2] - 1;
+  const bool bx = lc[0] > 0, by = lc[1] > 0, bz = lc[2] > 0;
   Spinor<float> xk = src;  // this site's current iterate
   const int napp = a.n_jac + (a.do_update ? 1 : 0);
   for (int it = 0; it < napp; ++it) {
-    float4* xb = cur ? xbuf1 : xbuf0;
-    float4* xnb = cur ? xbuf0 : xbuf1;
+    const bool more = it + 1 < napp;
     if (live) {
       zero(acc);
-      cs_intra_space<0>(a, xb, sl, lc, s, acc);
-      cs_intra_space<1>(a, xb, sl, lc, s, acc);
-      cs_intra_space<2>(a, xb, sl, lc, s, acc);
-      // t hops: the neighbouring slices' x (and, backward, their links)
-      // through distributed shared memory
-      if (lt < K - 1) {
-        const float4* rx = cl.map_shared_rank(xb, lt + 1);
-        Spinor<float> p;
-        cs_load_x(rx, S, s, p);
-        cs_hop<3, -1>(cs_link(sl, S, 3, s), p, 1.f, acc);
+      cs_intra_space<0>(xb, sl, S, s, 1, fx, bx, acc);
+      cs_intra_space<1>(xb, sl, S, s, a.sd[0], fy, by, acc);
+      cs_intra_space<2>(xb, sl, S, s, a.sd[0] * a.sd[1], fz, bz, acc);
+      HalfSpinor<float> h, uh;
+      if (above) {
+        cs_load_half(t_up, S, s, h);
+        su3_mul(cs_link(sl, S, 3, s), h, uh);
+        accumulate<3, -1>(acc, uh);
       }
-      if (lt > 0) {
-        const float4* rx = cl.map_shared_rank(xb, lt - 1);
-        const unsigned char* rl = cl.map_shared_rank(sl, lt - 1);
-        Spinor<float> p;
-        cs_load_x(rx, S, s, p);
-        cs_hop<3, +1>(cs_link(rl, S, 3, s), p, 1.f, acc);
+      if (below) {
+        cs_load_half(t_dn, S, s, uh);
+        accumulate<3, +1>(acc, uh);
       }
+    }
+    if (more) cs_arrive();  // this thread has read x and the half spinors
+    if (live) {
       cs_clover(sc, s, acc);
       if (it < a.n_jac) {
         // x_k = s + kappa C_inv H_cc x_{k-1}
@@ -317,7 +403,6 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
             xk.v[sp][c].re = fmaf(a.kappa, acc.v[sp][c].re, src.v[sp][c].re);
             xk.v[sp][c].im = fmaf(a.kappa, acc.v[sp][c].im, src.v[sp][c].im);
           }
-        cs_store_x(xnb, S, s, xk);
       } else {
         // s + b - x + kappa C_inv H_cc x
         Spinor<float> b;
@@ -334,13 +419,17 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
         a.s_out.store(g, dom, st, acc);
       }
     }
-    if (it < a.n_jac) {
-      cl.sync();  // every slice has read the old buffer and written the new one
-      cur ^= 1;
+    if (more) {
+      cs_wait_all();  // every slice has read the old x and half spinors
+      if (live) {
+        cs_store_x(xb, S + CS_GHOST, s, xk);
+        cs_push_t(below, above, sl, S, s, xk);
+      }
+      cs_arrive();
+      cs_wait_all();  // and now holds the new ones
     }
   }
   if (live) a.x.store(g, dom, st, xk);
-  cl.sync();  // the neighbours' last reads of this CTA's shared memory are done
 }
 
 // ---------------------------------------------------------------------------
@@ -440,9 +529,9 @@ void sap_cluster_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n
   a.extra_tx = ctx->inject == QCD_INJECT_STAGING_WAIT ? 16 : 0;
   const int K = a.sd[3];
   const int threads = (a.slice + 31) / 32 * 32;
-  const size_t smem = (size_t)CS_BYTES_PER_SITE * a.slice + 16;
+  const size_t smem = (size_t)CS_BYTES_PER_SITE * a.slice + CS_EXTRA_BYTES;
   QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((size_t)CS_BYTES_PER_SITE * CS_MAX_SLICE + 16)));
+                                      (int)((size_t)CS_BYTES_PER_SITE * CS_MAX_SLICE + CS_EXTRA_BYTES)));
   const size_t v4 = (size_t)a.g.vol * 6;
   for (int r = 0; r < nrhs; ++r) {
     a.b = F32Spinor{(float4*)b + r * v4};
