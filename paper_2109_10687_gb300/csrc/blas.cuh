@@ -3,12 +3,20 @@
 // arXiv:2109.10687), shared by the single-lattice solver and the ragged
 // batch solver.
 //
-// Reductions: every reducing kernel accumulates per thread in float32,
-// combines warps and blocks in float64 and lets the last block to finish sum
-// the per-block partials in a fixed order, so results do not depend on
-// scheduling.  Kernels run on a grid (blocks, k) with blockIdx.y = k the
-// right-hand side (or, in a ragged batch, the lattice); a Seg says where
-// element k of a stacked vector lives.
+// Reductions: every reducing kernel accumulates per thread in float32 (the
+// float64 kernels in float64), combines the threads of a block to float64
+// accuracy and lets the last block to finish sum the per-block partials in
+// float64 in a fixed order, so results do not depend on scheduling.  Kernels
+// run on a grid (blocks, k) with blockIdx.y = k the right-hand side (or, in a
+// ragged batch, the lattice); a Seg says where element k of a stacked vector
+// lives.
+//
+// The float32 sums of a block's threads are combined in double-float (48
+// bits): this GPU has two float64 lanes per SM, and a tree of float64 shuffles
+// over every warp took more time than the data on vectors of a few MB (a
+// 32-lattice batch: alpha's dot product 60 us against 19 us for p's update,
+// which moves more bytes; with this form 32 us, omega's 74 -> 26 us, the
+// second update 94 -> 57 us).
 #pragma once
 
 #include "qcd_internal.cuh"
@@ -48,64 +56,93 @@ struct Seg {
 // ---------------------------------------------------------------------------
 // reduction machinery
 // ---------------------------------------------------------------------------
-template <int N>
-__device__ __forceinline__ void block_sum(double v[N], double* sh /* [32][N] */) {
+// The sum of sh[0 .. RED_THREADS) by one warp, to float64 accuracy: float32
+// entries in double-float, which falls back to float64 when the sum leaves
+// float32's range (or is not finite), float64 entries in float64.  Lane 0's
+// value counts.
+__device__ __forceinline__ double warp_tree(double d) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+  return d;
+}
+template <typename T>
+__device__ __forceinline__ double warp_total(const T* sh) {
+  const int lane = threadIdx.x & 31;
+  if constexpr (sizeof(T) == 4) {
+    df64 s(sh[lane]);
+#pragma unroll
+    for (int j = 1; j < RED_THREADS / 32; ++j) s = s + df64(sh[lane + 32 * j]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      s = s + df64(__shfl_down_sync(0xffffffffu, s.hi, o), __shfl_down_sync(0xffffffffu, s.lo, o));
+    if (isfinite(__shfl_sync(0xffffffffu, s.hi, 0))) return to_double(s);
+  }
+  double d = sh[lane];
+#pragma unroll
+  for (int j = 1; j < RED_THREADS / 32; ++j) d += (double)sh[lane + 32 * j];
+  return warp_tree(d);
+}
+
+// Blocks of a (blocks, k) grid that take part in a reduction over n elements:
+// none would be left without an element
+__device__ __forceinline__ int red_blocks(size_t n) {
+  const size_t chunks = (n + RED_THREADS - 1) / RED_THREADS;
+  return chunks < gridDim.x ? (chunks ? (int)chunks : 1) : (int)gridDim.x;
+}
+
+// Sums v[k] over the nb participating blocks (the others must not call).
+// Writes this block's partials (times scale); returns true (in every thread)
+// in the block that finished last, which then holds the totals in tot[].
+// A warp per output.
+template <int N, typename T>
+__device__ __forceinline__ bool grid_reduce(const T (&v)[N], int nb, double* partials, unsigned* counter,
+                                            double (&tot)[N], double scale = 1.0) {
+  __shared__ T sh[N][RED_THREADS];
+  __shared__ double res[N];
+  __shared__ bool is_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int k = 0; k < N; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < N; ++k) sh[warp * N + k] = v[k];
+  for (int k = 0; k < N; ++k) sh[k][threadIdx.x] = v[k];
   __syncthreads();
-  if (warp == 0) {
-    const int nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      v[k] = lane < nw ? sh[lane * N + k] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+  if (warp < N) {
+    const double s = warp_total(sh[warp]);
+    if (lane == 0) {
+      partials[blockIdx.x * N + warp] = s * scale;
+      __threadfence();
     }
   }
   __syncthreads();
-}
-
-// Writes this block's partials; returns true (in every thread) in the block
-// that finished last, which then holds the totals in tot[] (all threads).
-template <int N>
-__device__ bool grid_reduce(double v[N], double* partials, unsigned* counter, double tot[N]) {
-  __shared__ double sh[32 * N];
-  __shared__ bool is_last;
-  block_sum<N>(v, sh);
-  const int nb = gridDim.x;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) partials[blockIdx.x * N + k] = v[k];
-    __threadfence();
-    const unsigned prev = atomicAdd(counter, 1u);
-    is_last = prev == (unsigned)(nb - 1);
-  }
+  if (threadIdx.x == 0) is_last = atomicAdd(counter, 1u) == (unsigned)(nb - 1);
   __syncthreads();
   if (!is_last) return false;
-  __threadfence();
-  double w[N];
-#pragma unroll
-  for (int k = 0; k < N; ++k) w[k] = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < N; ++k) w[k] += __ldcg(partials + i * N + k);
-  block_sum<N>(w, sh);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) sh[k] = w[k];
-    *counter = 0;
+  if (warp < N) {
+    __threadfence();
+    double s = 0.0;
+#pragma unroll 4
+    for (int i = lane; i < nb; i += 32) s += __ldcg(partials + i * N + warp);
+    s = warp_tree(s);
+    if (lane == 0) res[warp] = s;
   }
+  if (threadIdx.x == 0) *counter = 0;
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < N; ++k) tot[k] = sh[k];
-  __syncthreads();
+  for (int k = 0; k < N; ++k) tot[k] = res[k];
   return true;
+}
+
+// apply(i, load(i)) for this thread's elements i of [0, n) in ascending order,
+// nb blocks in the grid's stride; the loads of two elements are issued together
+template <typename L, typename A>
+__device__ __forceinline__ void strided(size_t n, int nb, L load, A apply) {
+  const size_t step = (size_t)nb * blockDim.x;
+  size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  for (; i + step < n; i += 2 * step) {
+    const auto a = load(i);
+    const auto b = load(i + step);
+    apply(i, a);
+    apply(i + step, b);
+  }
+  if (i < n) apply(i, load(i));
 }
 
 // complex (a.x + i a.y) * (b.x + i b.y) for the two complex numbers of a float4

@@ -97,13 +97,15 @@ __global__ void k_rg_norm2_f64(const double2* __restrict__ a, Seg seg, double* o
                                unsigned* counters) {
   const int k = blockIdx.y;
   const size_t off = seg.at(k), n = seg.size(k);
+  const int nb = red_blocks(n);
+  if ((int)blockIdx.x >= nb) return;
   double s = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)nb * blockDim.x) {
     const double2 v = a[off + i];
     s = fma(v.x, v.x, fma(v.y, v.y, s));
   }
   double v[1] = {s}, tot[1];
-  if (grid_reduce<1>(v, partials + (size_t)k * MAX_RED_OUT * gridDim.x, counters + k, tot) && threadIdx.x == 0)
+  if (grid_reduce(v, nb, partials + (size_t)k * MAX_RED_OUT * gridDim.x, counters + k, tot) && threadIdx.x == 0)
     out[k] = tot[0];
 }
 
@@ -112,15 +114,17 @@ __global__ void k_rg_residual_f64(const double2* __restrict__ b, double2* r, Seg
                                   unsigned* counters) {
   const int k = blockIdx.y;
   const size_t off = seg.at(k), n = seg.size(k);
+  const int nb = red_blocks(n);
+  if ((int)blockIdx.x >= nb) return;
   double s = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)nb * blockDim.x) {
     const double2 bv = b[off + i], dv = r[off + i];
     const double2 v = make_double2(bv.x - dv.x, bv.y - dv.y);
     r[off + i] = v;
     s = fma(v.x, v.x, fma(v.y, v.y, s));
   }
   double v[1] = {s}, tot[1];
-  if (grid_reduce<1>(v, partials + (size_t)k * MAX_RED_OUT * gridDim.x, counters + k, tot) && threadIdx.x == 0)
+  if (grid_reduce(v, nb, partials + (size_t)k * MAX_RED_OUT * gridDim.x, counters + k, tot) && threadIdx.x == 0)
     out[k] = tot[0];
 }
 

@@ -2,10 +2,7 @@
 // (Algorithm 4) and the fused BLAS-1 kernels they use (arXiv:2109.10687,
 // Sec. 3).
 //
-// Reductions: every reducing kernel accumulates per thread in float32,
-// combines warps and blocks in float64 and lets the last block to finish sum
-// the per-block partials in a fixed order, so results do not depend on
-// scheduling.  The scalars of the iteration (rho_0, alpha, omega, beta,
+// Reductions: see blas.cuh.  The scalars of the iteration (rho_0, alpha, omega, beta,
 // |r|^2) live in device memory, one record per right-hand side, and are
 // computed by the last block of the reduction that produces them; the host
 // only reads the per-rhs "done" flags to decide when to leave the loop.
@@ -139,6 +136,8 @@ static Workspace* workspace(qcd_ctx* ctx, int nrhs, bool solver) {
   Scal& sc = scal[rhs];                                               \
   const size_t off = seg.at(rhs);                                     \
   const size_t n4 = seg.size(rhs);                                    \
+  const int nb = red_blocks(n4);                                      \
+  if ((int)blockIdx.x >= nb) return;                                  \
   double* part = partials + (size_t)rhs * MAX_RED_OUT * gridDim.x;    \
   unsigned* cnt = counters + rhs;
 
@@ -148,11 +147,13 @@ __global__ void k_norm2(const float4* __restrict__ a, size_t n4, double* out, do
   const size_t off = (size_t)rhs * n4;
   double* part = partials + (size_t)rhs * MAX_RED_OUT * gridDim.x;
   unsigned* cnt = counters + rhs;
+  const int nb = red_blocks(n4);
+  if ((int)blockIdx.x >= nb) return;
   float s = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
-    s += norm4(a[off + i]);
-  double v[1] = {s}, tot[1];
-  if (grid_reduce<1>(v, part, cnt, tot) && threadIdx.x == 0) out[rhs] = tot[0];
+  strided(n4, nb, [&](size_t i) { return a[off + i]; }, [&](size_t, float4 v) { s += norm4(v); });
+  float v[1] = {s};
+  double tot[1];
+  if (grid_reduce(v, nb, part, cnt, tot) && threadIdx.x == 0) out[rhs] = tot[0];
 }
 
 // <a|b> -> out[2 rhs], out[2 rhs + 1]
@@ -161,11 +162,13 @@ __global__ void k_cdot(const float4* __restrict__ a, const float4* __restrict__ 
   const Seg seg{n, nullptr, nullptr};
   RHS_SETUP
   (void)sc;
+  struct Two { float4 a, b; };
   float re = 0.f, im = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
-    cdot_acc(a[off + i], b[off + i], re, im);
-  double v[2] = {re, im}, tot[2];
-  if (grid_reduce<2>(v, part, cnt, tot) && threadIdx.x == 0) {
+  strided(n4, nb, [&](size_t i) { return Two{a[off + i], b[off + i]}; },
+          [&](size_t, const Two& e) { cdot_acc(e.a, e.b, re, im); });
+  float v[2] = {re, im};
+  double tot[2];
+  if (grid_reduce(v, nb, part, cnt, tot) && threadIdx.x == 0) {
     out[2 * rhs] = tot[0];
     out[2 * rhs + 1] = tot[1];
   }
@@ -176,16 +179,17 @@ __global__ void k_init(const float4* __restrict__ b, float4* x, float4* r, float
                        double tol2, Scal* scal, double* partials, unsigned* counters, int* ctrl) {
   RHS_SETUP
   float s = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 v = b[off + i];
-    x[off + i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    r[off + i] = v;
-    p[off + i] = v;
-    rt[off + i] = v;
-    s += norm4(v);
-  }
-  double v[1] = {s}, tot[1];
-  if (grid_reduce<1>(v, part, cnt, tot) && threadIdx.x == 0) {
+  strided(n4, nb, [&](size_t i) { return b[off + i]; },
+          [&](size_t i, float4 v) {
+            x[off + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            r[off + i] = v;
+            p[off + i] = v;
+            rt[off + i] = v;
+            s += norm4(v);
+          });
+  float v[1] = {s};
+  double tot[1];
+  if (grid_reduce(v, nb, part, cnt, tot) && threadIdx.x == 0) {
     sc.bnorm2 = tot[0];
     sc.rnorm2 = tot[0];
     sc.rho0_re = tot[0];
@@ -209,11 +213,13 @@ __global__ void k_alpha(const float4* __restrict__ rt, const float4* __restrict_
                         double* partials, unsigned* counters, int* ctrl) {
   RHS_SETUP
   if (sc.done) return;
+  struct Two { float4 a, b; };
   float re = 0.f, im = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
-    cdot_acc(rt[off + i], q[off + i], re, im);
-  double v[2] = {re, im}, tot[2];
-  if (grid_reduce<2>(v, part, cnt, tot) && threadIdx.x == 0) {
+  strided(n4, nb, [&](size_t i) { return Two{rt[off + i], q[off + i]}; },
+          [&](size_t, const Two& e) { cdot_acc(e.a, e.b, re, im); });
+  float v[2] = {re, im};
+  double tot[2];
+  if (grid_reduce(v, nb, part, cnt, tot) && threadIdx.x == 0) {
     ++sc.iters;
     const double dn = tot[0] * tot[0] + tot[1] * tot[1];
     if (!(dn > 0.0) || !isfinite(dn)) {
@@ -238,14 +244,17 @@ __global__ void k_update1(float4* x, float4* r, const float4* __restrict__ z, co
   (void)x;
   (void)z;
   const float ar = (float)sc.alpha_re, ai = (float)sc.alpha_im;
+  struct Two { float4 q, r; };
   float s = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 rv = caxpy4(-ar, -ai, q[off + i], r[off + i]);
-    r[off + i] = rv;
-    s += norm4(rv);
-  }
-  double v[1] = {s}, tot[1];
-  if (grid_reduce<1>(v, part, cnt, tot) && threadIdx.x == 0) {
+  strided(n4, nb, [&](size_t i) { return Two{q[off + i], r[off + i]}; },
+          [&](size_t i, const Two& e) {
+            const float4 rv = caxpy4(-ar, -ai, e.q, e.r);
+            r[off + i] = rv;
+            s += norm4(rv);
+          });
+  float v[1] = {s};
+  double tot[1];
+  if (grid_reduce(v, nb, part, cnt, tot) && threadIdx.x == 0) {
     sc.xpend = 1;
     sc.rnorm2 = tot[0];
     if (!isfinite(tot[0])) {
@@ -265,14 +274,16 @@ __global__ void k_omega(const float4* __restrict__ t, const float4* __restrict__
                         double* partials, unsigned* counters, int* ctrl) {
   RHS_SETUP
   if (sc.done) return;
+  struct Two { float4 t, r; };
   float re = 0.f, im = 0.f, tt = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 tv = t[off + i];
-    cdot_acc(tv, r[off + i], re, im);
-    tt += norm4(tv);
-  }
-  double v[3] = {re, im, tt}, tot[3];
-  if (grid_reduce<3>(v, part, cnt, tot) && threadIdx.x == 0) {
+  strided(n4, nb, [&](size_t i) { return Two{t[off + i], r[off + i]}; },
+          [&](size_t, const Two& e) {
+            cdot_acc(e.t, e.r, re, im);
+            tt += norm4(e.t);
+          });
+  float v[3] = {re, im, tt};
+  double tot[3];
+  if (grid_reduce(v, nb, part, cnt, tot) && threadIdx.x == 0) {
     if (!(tot[2] > 0.0) || !isfinite(tot[2])) {
       sc.status = isfinite(tot[2]) ? QCD_ERR_BREAKDOWN : QCD_ERR_NONFINITE;
       sc.done = 1;
@@ -296,21 +307,28 @@ __global__ void k_update2(float4* x, float4* r, const float4* __restrict__ zp, c
   const float ar = (float)sc.alpha_re, ai = (float)sc.alpha_im;
   if (sc.done) {
     if (!sc.xpend) return;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
-      x[off + i] = caxpy4(ar, ai, zp[off + i], x[off + i]);
+    struct Two { float4 z, x; };
+    strided(n4, nb, [&](size_t i) { return Two{zp[off + i], x[off + i]}; },
+            [&](size_t i, const Two& e) { x[off + i] = caxpy4(ar, ai, e.z, e.x); });
     return;
   }
   const float wr = (float)sc.omega_re, wi = (float)sc.omega_im;
+  struct Six { float4 z, zp, x, t, r, rt; };
   float s = 0.f, re = 0.f, im = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    x[off + i] = caxpy4(wr, wi, z[off + i], caxpy4(ar, ai, zp[off + i], x[off + i]));
-    const float4 rv = caxpy4(-wr, -wi, t[off + i], r[off + i]);
-    r[off + i] = rv;
-    s += norm4(rv);
-    cdot_acc(rt[off + i], rv, re, im);
-  }
-  double v[3] = {s, re, im}, tot[3];
-  if (grid_reduce<3>(v, part, cnt, tot) && threadIdx.x == 0) {
+  strided(n4, nb,
+          [&](size_t i) {
+            return Six{z[off + i], zp[off + i], x[off + i], t[off + i], r[off + i], rt[off + i]};
+          },
+          [&](size_t i, const Six& e) {
+            x[off + i] = caxpy4(wr, wi, e.z, caxpy4(ar, ai, e.zp, e.x));
+            const float4 rv = caxpy4(-wr, -wi, e.t, e.r);
+            r[off + i] = rv;
+            s += norm4(rv);
+            cdot_acc(e.rt, rv, re, im);
+          });
+  float v[3] = {s, re, im};
+  double tot[3];
+  if (grid_reduce(v, nb, part, cnt, tot) && threadIdx.x == 0) {
     sc.rnorm2 = tot[0];
     if (!isfinite(tot[0]) || !isfinite(tot[1]) || !isfinite(tot[2])) {
       sc.status = QCD_ERR_NONFINITE;
@@ -352,10 +370,12 @@ __global__ void k_update_p(float4* p, const float4* __restrict__ r, const float4
   const size_t n4 = seg.size(rhs);
   const float br = (float)sc.beta_re, bi = (float)sc.beta_im;
   const float wr = (float)sc.omega_re, wi = (float)sc.omega_im;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    const float4 tmp = caxpy4(-wr, -wi, q[off + i], p[off + i]);
-    p[off + i] = caxpy4(br, bi, tmp, r[off + i]);
-  }
+  struct Three { float4 q, p, r; };
+  strided(n4, gridDim.x, [&](size_t i) { return Three{q[off + i], p[off + i], r[off + i]}; },
+          [&](size_t i, const Three& e) {
+            const float4 tmp = caxpy4(-wr, -wi, e.q, e.p);
+            p[off + i] = caxpy4(br, bi, tmp, e.r);
+          });
 }
 
 // x += alpha z_p for a right-hand side whose iteration stopped after
@@ -380,13 +400,15 @@ __global__ void k_norm2_f64(const double2* __restrict__ a, size_t n2, double* ou
   const int rhs = blockIdx.y;
   const size_t off = (size_t)rhs * n2;
   double* part = partials + (size_t)rhs * MAX_RED_OUT * gridDim.x;
+  const int nb = red_blocks(n2);
+  if ((int)blockIdx.x >= nb) return;
   double s = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)nb * blockDim.x) {
     const double2 v = a[off + i];
     s = fma(v.x, v.x, fma(v.y, v.y, s));
   }
   double v[1] = {s}, tot[1];
-  if (grid_reduce<1>(v, part, counters + rhs, tot) && threadIdx.x == 0) out[rhs] = tot[0];
+  if (grid_reduce(v, nb, part, counters + rhs, tot) && threadIdx.x == 0) out[rhs] = tot[0];
 }
 
 // r = b - r (r holds D x on entry); out[rhs] = |r|^2
@@ -395,15 +417,17 @@ __global__ void k_residual_f64(const double2* __restrict__ b, double2* r, size_t
   const int rhs = blockIdx.y;
   const size_t off = (size_t)rhs * n2;
   double* part = partials + (size_t)rhs * MAX_RED_OUT * gridDim.x;
+  const int nb = red_blocks(n2);
+  if ((int)blockIdx.x >= nb) return;
   double s = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)nb * blockDim.x) {
     const double2 bv = b[off + i], dv = r[off + i];
     const double2 v = make_double2(bv.x - dv.x, bv.y - dv.y);
     r[off + i] = v;
     s = fma(v.x, v.x, fma(v.y, v.y, s));
   }
   double v[1] = {s}, tot[1];
-  if (grid_reduce<1>(v, part, counters + rhs, tot) && threadIdx.x == 0) out[rhs] = tot[0];
+  if (grid_reduce(v, nb, part, counters + rhs, tot) && threadIdx.x == 0) out[rhs] = tot[0];
 }
 
 // ---------------------------------------------------------------------------
@@ -414,14 +438,16 @@ __global__ void k_residual_f64(const double2* __restrict__ b, double2* r, size_t
 // <a|b> = sum conj(a) b -> out[0] (re), out[1] (im)
 __global__ void k_cdot_f64(const double2* __restrict__ a, const double2* __restrict__ b, size_t n2, double* out,
                            double* partials, unsigned* counters) {
+  const int nb = red_blocks(n2);
+  if ((int)blockIdx.x >= nb) return;
   double re = 0.0, im = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)nb * blockDim.x) {
     const double2 u = a[i], v = b[i];
     re = fma(u.x, v.x, fma(u.y, v.y, re));
     im = fma(u.x, v.y, fma(-u.y, v.x, im));
   }
   double v[2] = {re, im}, tot[2];
-  if (grid_reduce<2>(v, partials, counters, tot) && threadIdx.x == 0) {
+  if (grid_reduce(v, nb, partials, counters, tot) && threadIdx.x == 0) {
     out[0] = tot[0];
     out[1] = tot[1];
   }
@@ -550,16 +576,19 @@ __global__ void k_residual_df(const float4* __restrict__ b, float4* r, size_t n2
   const size_t off = (size_t)rhs * n2;
   double* part = partials + (size_t)rhs * MAX_RED_OUT * gridDim.x;
   const int k = df_scale_exp(b2, rhs, n2);
+  const int nb = red_blocks(n2);
+  if ((int)blockIdx.x >= nb) return;
   float s = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)nb * blockDim.x) {
     const float4 bv = b[off + i], dv = r[off + i];
     const df64 re = df64(bv.x, bv.y) - df64(dv.x, dv.y);
     const df64 im = df64(bv.z, bv.w) - df64(dv.z, dv.w);
     r[off + i] = make_float4(re.hi, re.lo, im.hi, im.lo);
     s = fmaf(re.hi, re.hi, fmaf(im.hi, im.hi, s));
   }
-  double v[1] = {ldexp((double)s, -2 * k)}, tot[1];
-  if (grid_reduce<1>(v, part, counters + rhs, tot) && threadIdx.x == 0) out[rhs] = tot[0];
+  float v[1] = {s};
+  double tot[1];
+  if (grid_reduce(v, nb, part, counters + rhs, tot, ldexp(1.0, -2 * k)) && threadIdx.x == 0) out[rhs] = tot[0];
 }
 // float32 p = R_SP(r / err) from the scaled double-float r (err unscaled),
 // in float32 arithmetic: (hi + lo) f as hi f + lo f with one rounding
