@@ -148,11 +148,27 @@ def _on_device(t):
     return 0 if isinstance(t, np.ndarray) else int(t.is_cuda)
 
 
+def _current_stream_raw():
+    """() -> raw handle of torch's current CUDA stream.  torch builds a Stream
+    object on every public query, several microseconds of an operator call on
+    a small lattice; its own code generators use the raw query."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(torch.cuda.current_device())
+
+
+_raw_stream = None
+
+
 def _stream(stream):
+    global _raw_stream
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
-    import torch
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None:
+        _raw_stream = _current_stream_raw()
+    return _raw_stream()
 
 
 def check(ctx, rc):

@@ -312,89 +312,74 @@ extern "C" int qcd_grad(qcd_ctx* ctx, const double* eta, const double* b, const 
     QCD_REQUIRE((x || b) && (lam || eta), QCD_ERR_ARG, "qcd_grad: need b or x, and eta or lambda");
     const Geom& g = ctx->geom;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t cbytes = (size_t)g.vol * 24 * sizeof(double);
-    double *xs = nullptr, *ls = nullptr;
-    float4 *x32 = nullptr, *l32 = nullptr;
-    float2* V = nullptr;
-    struct Guard {
-      void* p[6];
-      ~Guard() {
-        for (void* q : p)
-          if (q) cudaFree(q);
-      }
-    } guard{{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}};
-    QCD_CUDA_CHECK(cudaMalloc(&xs, cbytes));
-    guard.p[0] = xs;
-    QCD_CUDA_CHECK(cudaMalloc(&ls, cbytes));
-    guard.p[1] = ls;
+    const size_t fdoubles = (size_t)g.vol * 24;  // one canonical field
+    const size_t cbytes = fdoubles * sizeof(double);
+    const size_t b32 = spinor_bytes(g, QCD_PREC_SINGLE);
     qcd_solve_params P;
     if (params) P = *params;
     else qcd_solve_params_default(&P);
     P.x_is_guess = 0;
     qcd_solve_info info;
     const int pb = ctx->basis == QCD_BASIS_PAPER;
-    if (!x && !lam && P.outer_restart == 0) {
-      // both solves at once: D [x, y] = [b, gamma_5 eta] as two right-hand
-      // sides of one batched solve (every launch serves both), lambda = gamma_5 y
-      double *rhs2 = nullptr, *sol2 = nullptr;
-      QCD_CUDA_CHECK(cudaMalloc(&rhs2, 2 * cbytes));
-      guard.p[4] = rhs2;
-      QCD_CUDA_CHECK(cudaMalloc(&sol2, 2 * cbytes));
-      guard.p[5] = sol2;
-      QCD_CUDA_CHECK(cudaMemcpyAsync(rhs2, b, cbytes, cudaMemcpyDeviceToDevice, st));
-      QCD_CUDA_CHECK(cudaMemcpyAsync(rhs2 + (size_t)g.vol * 24, eta, cbytes, cudaMemcpyDeviceToDevice, st));
-      gamma5_canonical_kernel<<<grid_for(g.vol, 256), 256, 0, st>>>(g.vol, rhs2 + (size_t)g.vol * 24, pb);
+    const int with_clover = ctx->csw != 0.0;
+    // one solve of two right-hand sides when both x and lambda are missing
+    const bool both = !x && !lam && P.outer_restart == 0;
+    // Scratch in one buffer kept in the context (cudaMalloc and cudaFree of its
+    // parts took 0.5 ms of a 16^4 call): canonical sources and solutions of
+    // the solves, then the float32 fields and V of the force.
+    const size_t n_src = both ? 2 : (lam ? 0 : 1), n_sol = both ? 2 : (x ? 0 : 1) + (lam ? 0 : 1);
+    const size_t force_bytes = grad_U ? 2 * b32 + (with_clover ? (size_t)g.vol * 54 * sizeof(float2) : 0) : 0;
+    const size_t need = (n_src + n_sol) * cbytes + force_bytes;
+    if (need > ctx->grad_bytes) {
+      if (ctx->grad_buf) QCD_CUDA_CHECK(cudaFree(ctx->grad_buf));
+      ctx->grad_buf = nullptr;
+      ctx->grad_bytes = 0;
+      QCD_CUDA_CHECK(cudaMalloc(&ctx->grad_buf, need));
+      ctx->grad_bytes = need;
+    }
+    double* src = static_cast<double*>(ctx->grad_buf);
+    double* sol = src + n_src * fdoubles;
+    float4* x32 = reinterpret_cast<float4*>(sol + n_sol * fdoubles);
+    float4* l32 = x32 + b32 / sizeof(float4);
+    float2* V = reinterpret_cast<float2*>(l32 + b32 / sizeof(float4));
+    auto gamma5 = [&](double* f) {
+      gamma5_canonical_kernel<<<grid_for(g.vol, 256), 256, 0, st>>>(g.vol, f, pb);
       check_launch();
       ctx->launches++;
-      const int rc = qcd_solve(ctx, sol2, rhs2, 2, 1, &P, &info, stream);
+    };
+    const double *xs = x, *ls = lam;  // canonical x and lambda
+    if (both) {
+      // D [x, y] = [b, gamma_5 eta] (every launch serves both), lambda = gamma_5 y
+      QCD_CUDA_CHECK(cudaMemcpyAsync(src, b, cbytes, cudaMemcpyDeviceToDevice, st));
+      QCD_CUDA_CHECK(cudaMemcpyAsync(src + fdoubles, eta, cbytes, cudaMemcpyDeviceToDevice, st));
+      gamma5(src + fdoubles);
+      const int rc = qcd_solve(ctx, sol, src, 2, 1, &P, &info, stream);
       if (rc != QCD_OK) throw Error{rc, "qcd_grad: solve failed: " + ctx->err};
-      QCD_CUDA_CHECK(cudaMemcpyAsync(xs, sol2, cbytes, cudaMemcpyDeviceToDevice, st));
-      QCD_CUDA_CHECK(cudaMemcpyAsync(ls, sol2 + (size_t)g.vol * 24, cbytes, cudaMemcpyDeviceToDevice, st));
-      gamma5_canonical_kernel<<<grid_for(g.vol, 256), 256, 0, st>>>(g.vol, ls, pb);
-      check_launch();
-      ctx->launches++;
-      cudaFree(rhs2);
-      cudaFree(sol2);
-      guard.p[4] = guard.p[5] = nullptr;
+      xs = sol;
+      gamma5(sol + fdoubles);
+      ls = sol + fdoubles;
     } else {
-    if (x) {
-      QCD_CUDA_CHECK(cudaMemcpyAsync(xs, x, cbytes, cudaMemcpyDeviceToDevice, st));
-    } else {
-      const int rc = qcd_solve(ctx, xs, b, 1, 1, &P, &info, stream);
-      if (rc != QCD_OK) throw Error{rc, "qcd_grad: forward solve failed: " + ctx->err};
+      if (!x) {
+        const int rc = qcd_solve(ctx, sol, b, 1, 1, &P, &info, stream);
+        if (rc != QCD_OK) throw Error{rc, "qcd_grad: forward solve failed: " + ctx->err};
+        xs = sol;
+      }
+      if (!lam) {
+        double* l = sol + (x ? 0 : fdoubles);
+        QCD_CUDA_CHECK(cudaMemcpyAsync(src, eta, cbytes, cudaMemcpyDeviceToDevice, st));
+        gamma5(src);
+        const int rc = qcd_solve(ctx, l, src, 1, 1, &P, &info, stream);
+        if (rc != QCD_OK) throw Error{rc, "qcd_grad: adjoint solve failed: " + ctx->err};
+        gamma5(l);
+        ls = l;
+      }
     }
-    if (lam) {
-      QCD_CUDA_CHECK(cudaMemcpyAsync(ls, lam, cbytes, cudaMemcpyDeviceToDevice, st));
-    } else {
-      double* e5 = nullptr;
-      QCD_CUDA_CHECK(cudaMalloc(&e5, cbytes));
-      guard.p[4] = e5;
-      QCD_CUDA_CHECK(cudaMemcpyAsync(e5, eta, cbytes, cudaMemcpyDeviceToDevice, st));
-      gamma5_canonical_kernel<<<grid_for(g.vol, 256), 256, 0, st>>>(g.vol, e5, pb);
-      check_launch();
-      ctx->launches++;
-      const int rc = qcd_solve(ctx, ls, e5, 1, 1, &P, &info, stream);
-      if (rc != QCD_OK) throw Error{rc, "qcd_grad: adjoint solve failed: " + ctx->err};
-      gamma5_canonical_kernel<<<grid_for(g.vol, 256), 256, 0, st>>>(g.vol, ls, pb);
-      check_launch();
-      ctx->launches++;
-    }
-    }
-    if (grad_b) QCD_CUDA_CHECK(cudaMemcpyAsync(grad_b, ls, cbytes, cudaMemcpyDeviceToDevice, st));
     if (grad_U) {
-      const size_t b32 = spinor_bytes(g, QCD_PREC_SINGLE);
-      QCD_CUDA_CHECK(cudaMalloc(&x32, b32));
-      guard.p[2] = x32;
-      QCD_CUDA_CHECK(cudaMalloc(&l32, b32));
-      guard.p[3] = l32;
       int rc = qcd_import_spinor(ctx, x32, xs, QCD_PREC_SINGLE, 1, 1, stream);
       if (rc != QCD_OK) throw Error{rc, ctx->err};
       rc = qcd_import_spinor(ctx, l32, ls, QCD_PREC_SINGLE, 1, 1, stream);
       if (rc != QCD_OK) throw Error{rc, ctx->err};
-      const int with_clover = ctx->csw != 0.0;
       if (with_clover) {
-        QCD_CUDA_CHECK(cudaMalloc(&V, (size_t)g.vol * 54 * sizeof(float2)));
-        guard.p[5] = V;
         LaunchScope ls_(ctx, QCD_KC_OTHER, st);
         clover_v_kernel<<<grid_for(g.vol, 128), 128, 0, st>>>(g, F32Spinor{x32}, F32Spinor{l32},
                                                               (float)(ctx->kappa * ctx->csw), V);
@@ -408,6 +393,8 @@ extern "C" int qcd_grad(qcd_ctx* ctx, const double* eta, const double* b, const 
         check_launch();
       }
     }
+    // last: grad_b may be the caller's x or lambda
+    if (grad_b && grad_b != ls) QCD_CUDA_CHECK(cudaMemcpyAsync(grad_b, ls, cbytes, cudaMemcpyDeviceToDevice, st));
     QCD_CUDA_CHECK(cudaStreamSynchronize(st));
   } catch (const qcd::Error& e) {
     ctx->err = e.msg;

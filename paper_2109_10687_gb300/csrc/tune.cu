@@ -49,18 +49,28 @@ int tune_pick(qcd_ctx* ctx, const char* key, int nvariants, const char* const* n
   cudaEvent_t a, b;
   QCD_CUDA_CHECK(cudaEventCreate(&a));
   QCD_CUDA_CHECK(cudaEventCreate(&b));
-  int best_v = 0;
+  int best_v = 0, runs = 0;
   float best_ms = 1e30f;
   std::string all;
   for (int v = 0; v < nvariants; ++v) {
+    // a variant of a kernel that is not short is timed once first, and twice
+    // more only if it is not far behind the best so far (the first call pays
+    // for all of them)
+    auto timed = [&](int n) {
+      QCD_CUDA_CHECK(cudaEventRecord(a, st));
+      for (int r = 0; r < n; ++r) run(v);
+      QCD_CUDA_CHECK(cudaEventRecord(b, st));
+      QCD_CUDA_CHECK(cudaEventSynchronize(b));
+      float t = 0.f;
+      QCD_CUDA_CHECK(cudaEventElapsedTime(&t, a, b));
+      runs += n;
+      return t / n;
+    };
     run(v);  // warm-up
-    QCD_CUDA_CHECK(cudaEventRecord(a, st));
-    for (int r = 0; r < 3; ++r) run(v);
-    QCD_CUDA_CHECK(cudaEventRecord(b, st));
-    QCD_CUDA_CHECK(cudaEventSynchronize(b));
-    float ms = 0.f;
-    QCD_CUDA_CHECK(cudaEventElapsedTime(&ms, a, b));
-    ms /= 3.f;
+    ++runs;
+    const bool probe = v > 0 && best_ms > 0.05f;
+    float ms = probe ? timed(1) : 0.f;
+    if (ms <= 1.3f * best_ms) ms = timed(probe ? 2 : 3);
     char item[96];
     std::snprintf(item, sizeof item, "%s%s %.4f", v ? ", " : "", names ? names[v] : std::to_string(v).c_str(), ms);
     all += item;
@@ -71,7 +81,7 @@ int tune_pick(qcd_ctx* ctx, const char* key, int nvariants, const char* const* n
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
-  ctx->launches += 4LL * nvariants;
+  ctx->launches += runs;
   t->best[key] = {best_v, best_ms, names ? names[best_v] : std::to_string(best_v), all};
   return best_v;
 }
