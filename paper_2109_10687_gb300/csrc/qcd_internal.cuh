@@ -778,9 +778,10 @@ inline int grid_for(long long n, int block) { return (int)((n + block - 1) / blo
 // Autotuner: returns the launch variant to use for `key`.  The first call per
 // key with tuning on (and outside stream capture) times every variant with
 // CUDA events -- run(v) must be an out-of-place launch whose repetition is
-// harmless -- and remembers the fastest; later calls return it.
+// harmless -- and remembers the fastest; later calls return it.  A key never
+// timed gets the variant `untuned`.
 int tune_pick(qcd_ctx* ctx, const char* key, int nvariants, const char* const* names,
-              const std::function<void(int)>& run, cudaStream_t st);
+              const std::function<void(int)>& run, cudaStream_t st, int untuned = 0);
 void tuner_free(qcd_ctx* ctx);
 
 // internal entry points implemented in the other translation units
@@ -789,6 +790,10 @@ void tuner_free(qcd_ctx* ctx);
 // the solver, where it measured slower
 void dslash_launch(qcd_ctx* ctx, void* out, const void* in, int prec, int mode, int nrhs, cudaStream_t st,
                    bool pdl = false);
+// the float32 operators on several right-hand sides of 4^4 blocks (dslash_mrhs.cu)
+bool dslash_mrhs_fits(const Geom& g, int nrhs);
+void dslash_mrhs_launch(qcd_ctx* ctx, void* out, const void* in, int mode, int nrhs, bool use12, cudaStream_t st,
+                        bool pdl);
 void clover_apply_launch(qcd_ctx* ctx, void* out, const void* in, int prec, int inverse, int nrhs,
                          cudaStream_t st);
 void ablock_launch(qcd_ctx* ctx, float4* out, const float4* in, int row, int col, cudaStream_t st);

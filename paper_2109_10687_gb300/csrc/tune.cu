@@ -39,13 +39,13 @@ void tuner_free(qcd_ctx* ctx) {
 }
 
 int tune_pick(qcd_ctx* ctx, const char* key, int nvariants, const char* const* names,
-              const std::function<void(int)>& run, cudaStream_t st) {
+              const std::function<void(int)>& run, cudaStream_t st, int untuned) {
   Tuner* t = tuner_of(ctx);
   auto it = t->best.find(key);
   if (it != t->best.end()) return it->second.variant;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(st, &cs);
-  if (!t->enabled || cs != cudaStreamCaptureStatusNone || nvariants <= 1) return 0;
+  if (!t->enabled || cs != cudaStreamCaptureStatusNone || nvariants <= 1) return untuned;
   cudaEvent_t a, b;
   QCD_CUDA_CHECK(cudaEventCreate(&a));
   QCD_CUDA_CHECK(cudaEventCreate(&b));
