@@ -833,13 +833,13 @@ void workspace_reset_graphs(qcd_ctx* ctx);
 // sites on the one-CTA kernel, larger ones on the cluster kernel)
 bool sap_domain_valid(const int dims[4], const int sdom[4]);
 void sap_general_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n_sap, int n_jac, int sap_prec,
-                       void* ws_s, cudaStream_t st);
+                       void* ws_s, void* halo, cudaStream_t st);
 // the same with one thread-block cluster per domain (float16 links and C_inv staged in shared memory)
 bool sap_cluster_eligible(const qcd_ctx* ctx, int sap_prec);
 bool sap_cluster_fits(const int sdom[4]);
 bool sap_general_fits(const int sdom[4]);  // the one-CTA kernel: at most 1152 sites
 void sap_cluster_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n_sap, int n_jac, void* ws_s,
-                       cudaStream_t st);
+                       void* halo, cudaStream_t st);
 void gauge_import_launch(qcd_ctx* ctx, const double* u, cudaStream_t st);
 
 // dslash modes

@@ -22,15 +22,16 @@
 namespace qcd {
 
 // x = M_SAP b for nrhs stacked float32 fields.  ws_s holds s (float32 or
-// float16), halo the block kernel's face halo (96 bytes per site); both are
-// sized for nrhs right-hand sides, which go through every launch together.
+// float16), halo the block and cluster kernels' face halo (96 bytes per site);
+// both are sized for nrhs right-hand sides, which go through every launch
+// together.
 // Domains set apart from the storage blocks have kernels of their own; 4^4
 // storage blocks take the block kernel (which on small lattices may hand over
 // to the split one), all others the kernel of sap_block.cu.
 void sap_apply_launch(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n_sap, int n_jac, int sap_prec,
                       void* ws_s, void* halo, cudaStream_t st) {
   if (ctx->sap_general) {
-    sap_general_apply(ctx, x, b, nrhs, n_sap, n_jac, sap_prec, ws_s, st);
+    sap_general_apply(ctx, x, b, nrhs, n_sap, n_jac, sap_prec, ws_s, halo, st);
     return;
   }
   const bool staged = sap_staged_available(ctx);

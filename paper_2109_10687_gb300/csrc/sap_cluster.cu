@@ -18,18 +18,26 @@
 // wait after the C_inv multiply) separates the reads of x and of the half
 // spinors from the next writes, the second those writes from the next reads.
 //
-// The surface term (hops that leave the domain) reads the other colour's x
-// and the neighbouring domains' links from memory; its lines are prefetched
-// to L1 while the staging copies are under way.  (One CTA fills an SM, so an
-// early start of the next launch would gain nothing; without it L1 holds no
-// line of an earlier launch.)
+// The surface term (hops that leave the domain): at the end of a launch every
+// site on a face leaves its half spinor for the neighbouring domain in a halo
+// in memory (cs_slot), from registers and the staged link; the next launch
+// reads one half spinor per face site, all of them in flight while the staging
+// copies are under way.  Domains whose faces need more than the caller's 96
+// bytes per site (extents of one) read the neighbours' x and links in place.
+//
+// The next launch may start early (programmatic dependent launch): its first
+// clusters take the SMs that the last wave of clusters leaves idle and bring
+// their operator in, then wait for this launch.  So whatever changes between
+// launches is read past L1.
 //
 // What bounds it: one CTA of 12 warps per SM (16x6x4x3: 190 KB of shared
-// memory), so each warp's chain of loads and multiply-adds.  Reading the
-// t neighbours' spinors and links from the other CTAs in place, with a branch
-// per hop, a sweep took 6.7 us for the clusters resident at a time and the rest
-// of a launch 13 us; now 3.8 and 12.7 us (32x24x16x24, 128 clusters in three
-// waves: a half-sweep with n_jac 2 96 -> 70 us).
+// memory), so each warp's chain of loads and multiply-adds, and whole waves
+// of clusters.  32x24x16x24, 128 clusters in three waves, a half-sweep with
+// n_jac 2: 96 us with the t neighbours' spinors and links read from the other
+// CTAs in place and a branch per hop; 70 with half spinors pushed there; 67
+// with the halo (before, the surface hops gathered x and links from memory);
+// 59 with early starts.  Of those 35 are the three sweeps.
+// M_SAP (n_sap 4, n_jac 2) 1000 -> 628 us.
 
 #include <cooperative_groups.h>
 
@@ -57,7 +65,11 @@ struct ClusterSapArgs {
   int colour, n_jac, do_surface, do_update;
   float kappa;
   F32Spinor s_in, s_out, x, b;
-  LinkPtrHalf U16;             // links in the internal layout (backward hops that enter the domain)
+  LinkPtrHalf U16;             // links in the internal layout (backward hops that enter the domain, without halo)
+  float4* halo;                // half spinors at the faces between domains, see cs_slot
+  size_t halo_at[4];           // where direction mu's begin
+  int face[4];                 // sites of a face of a domain
+  int do_halo;                 // leave the neighbours' half spinors (0 in the last launch)
   const unsigned char* links;  // staging: [domain][slice][mu][site][10 half2]
   const unsigned char* clov;   // staging: [domain][slice][site][9 uint4]
   int* status;
@@ -127,6 +139,15 @@ __device__ __forceinline__ void cs_store_x(float4* buf, int stride, int s, const
     buf[k * stride + s] = make_float4(a0.re, a0.im, a1.re, a1.im);
   }
 }
+// a field's site from memory, past L1 (an earlier launch wrote it)
+__device__ __forceinline__ void cs_read_x(const Geom& g, const F32Spinor& f, int dom, int s, Spinor<float>& a) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const float4 v = __ldcg(f.p + f.idx(g, dom, k, s));
+    a.v[(2 * k) / 3][(2 * k) % 3] = make_cx(v.x, v.y);
+    a.v[(2 * k + 1) / 3][(2 * k + 1) % 3] = make_cx(v.z, v.w);
+  }
+}
 // half spinors: float4 [3][slice]
 __device__ __forceinline__ void cs_load_half(const float4* buf, int slice, int s, HalfSpinor<float>& h) {
 #pragma unroll
@@ -185,6 +206,73 @@ __device__ __forceinline__ void cs_push_t(float4* below, float4* above, const un
 __device__ __forceinline__ void cs_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cs_wait_all() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
+// Half spinors between domains: float4 [direction][domain][3][face site], one
+// slot per site of the face between a domain and the next one up.  The lower
+// domain leaves U^dag P+ x there, the finished hop backward of the upper one,
+// which in its own launch leaves P- x, to be multiplied by the lower one's
+// link.  Either way the thread that reads a slot at the start of a launch is
+// the one that writes it at the end, and no other touches it in that launch.
+// At most 96 bytes per site as long as the extents' reciprocals sum to two.
+__device__ __forceinline__ float4* cs_slot(const ClusterSapArgs& a, const int D[4], long long jd, const int lc[4],
+                                           int mu, bool up) {
+  long long step = 1;
+  int f = 0, m = 1;
+#pragma unroll
+  for (int nu = 0; nu < 4; ++nu) {
+    if (nu < mu) step *= a.snd[nu];
+    if (nu == mu) continue;
+    f += m * lc[nu];
+    m *= a.sd[nu];
+  }
+  if (!up) jd += D[mu] == 0 ? (a.snd[mu] - 1) * step : -step;
+  return a.halo + a.halo_at[mu] + (size_t)jd * 3 * a.face[mu] + f;
+}
+// a slot, past L1: the launch before wrote it
+__device__ __forceinline__ void cs_read_slot(const float4* p, int face, HalfSpinor<float>& h) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float4 v = __ldcg(p + k * face);
+    h.h[(2 * k) / 3][(2 * k) % 3] = make_cx(v.x, v.y);
+    h.h[(2 * k + 1) / 3][(2 * k + 1) % 3] = make_cx(v.z, v.w);
+  }
+}
+// the half spinor of direction mu that a site on either face (upper first)
+// takes in; read long before it is used
+__device__ __forceinline__ void cs_halo_read(const ClusterSapArgs& a, const int D[4], long long jd, const int lc[4],
+                                             int mu, HalfSpinor<float>& h) {
+  const bool up = lc[mu] == a.sd[mu] - 1;
+  if (up || lc[mu] == 0) cs_read_slot(cs_slot(a, D, jd, lc, mu, up), a.face[mu], h);
+}
+template <int MU>
+__device__ __forceinline__ void cs_halo_in(const ClusterSapArgs& a, const unsigned char* sl, const int D[4],
+                                           long long jd, const int X[4], const int lc[4], int s,
+                                           const HalfSpinor<float>& in, Spinor<float>& acc) {
+  HalfSpinor<float> uh;
+  const bool up = lc[MU] == a.sd[MU] - 1;
+  if (up) {
+    su3_mul(cs_link(sl, a.slice, MU, s), in, uh);
+    accumulate<MU, -1>(acc, uh, (MU == 3 && X[3] + 1 == a.g.L[3]) ? (float)a.g.bc_t : 1.f);
+  }
+  if (lc[MU] == 0) {
+    if (up) cs_read_slot(cs_slot(a, D, jd, lc, MU, false), a.face[MU], uh);  // an extent of one: both faces
+    else uh = in;
+    accumulate<MU, +1>(acc, uh, (MU == 3 && X[3] == 0) ? (float)a.g.bc_t : 1.f);
+  }
+}
+template <int MU>
+__device__ __forceinline__ void cs_halo_out(const ClusterSapArgs& a, const unsigned char* sl, const int D[4],
+                                            long long jd, const int lc[4], int s, const Spinor<float>& x) {
+  HalfSpinor<float> h, uh;
+  if (lc[MU] == a.sd[MU] - 1) {
+    project<MU, +1>(x, h);
+    su3_dag_mul(cs_link(sl, a.slice, MU, s), h, uh);
+    cs_store_half(cs_slot(a, D, jd, lc, MU, true), a.face[MU], 0, uh);
+  }
+  if (lc[MU] == 0) {
+    project<MU, -1>(x, h);
+    cs_store_half(cs_slot(a, D, jd, lc, MU, false), a.face[MU], 0, h);
+  }
+}
 // L1 prefetch of what cs_inter reads for one hop: the spinor and, for a
 // backward hop, the neighbouring domain's link
 __device__ __forceinline__ void cs_prefetch(const ClusterSapArgs& a, const int Y[4], int mu, bool bwd) {
@@ -265,6 +353,7 @@ __device__ __forceinline__ bool cs_wait(uint64_t* bar) {
   return false;
 }
 
+template <bool HALO>
 __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSapArgs a) {
   extern __shared__ __align__(128) unsigned char csm[];
   const Geom& g = a.g;
@@ -279,8 +368,10 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
   unsigned char* sc = sl + 4 * CS_LINK_H2 * 4 * S;  // C_inv
   uint64_t* bar = reinterpret_cast<uint64_t*>(sc + CS_CLOV_U4 * 16 * S);
   int* bad = reinterpret_cast<int*>(bar + 1);
-  // the same decision in every CTA of the cluster: the flag was written before this launch
+  // the same decision in every CTA of the cluster: the flag was written before
+  // the first launch of the sequence, which is no early one
   if (loop_idle(g)) return;
+  if (HALO) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int tid = threadIdx.x;
   const bool live = tid < S;
   const int s = live ? tid : 0;
@@ -324,10 +415,20 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
   coords_to_internal(g, X, dom, st);
   for (int i = tid; i < 6 * CS_GHOST; i += blockDim.x)
     xb[(i / CS_GHOST) * (S + CS_GHOST) + S + i % CS_GHOST] = make_float4(0.f, 0.f, 0.f, 0.f);
+  // links and C_inv are constant; everything from here on is not
+  if (HALO) asm volatile("griddepcontrol.wait;" ::: "memory");
+  HalfSpinor<float> hin[4];
   Spinor<float> src;
   if (live) {
-    if (a.do_surface) cs_prefetch_surface(a, X, lc);
-    a.s_in.load(g, dom, st, src);
+    if (a.do_surface) {
+      if (HALO) {
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) cs_halo_read(a, D, jd, lc, mu, hin[mu]);
+      } else {
+        cs_prefetch_surface(a, X, lc);
+      }
+    }
+    cs_read_x(g, a.s_in, dom, st, src);
   }
   __syncthreads();  // barrier initialisation visible to every thread
   {
@@ -348,10 +449,17 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
   Spinor<float> acc;
   if (a.do_surface && live) {
     zero(acc);
-    cs_inter<0>(a, sl, X, lc, s, acc);
-    cs_inter<1>(a, sl, X, lc, s, acc);
-    cs_inter<2>(a, sl, X, lc, s, acc);
-    if (lt == K - 1 || lt == 0) cs_inter<3>(a, sl, X, lc, s, acc);
+    if (HALO) {
+      cs_halo_in<0>(a, sl, D, jd, X, lc, s, hin[0], acc);
+      cs_halo_in<1>(a, sl, D, jd, X, lc, s, hin[1], acc);
+      cs_halo_in<2>(a, sl, D, jd, X, lc, s, hin[2], acc);
+      if (lt == K - 1 || lt == 0) cs_halo_in<3>(a, sl, D, jd, X, lc, s, hin[3], acc);
+    } else {
+      cs_inter<0>(a, sl, X, lc, s, acc);
+      cs_inter<1>(a, sl, X, lc, s, acc);
+      cs_inter<2>(a, sl, X, lc, s, acc);
+      if (lt == K - 1 || lt == 0) cs_inter<3>(a, sl, X, lc, s, acc);
+    }
     cs_clover(sc, s, acc);
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp)
@@ -406,7 +514,7 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
       } else {
         // s + b - x + kappa C_inv H_cc x
         Spinor<float> b;
-        a.b.load(g, dom, st, b);
+        cs_read_x(g, a.b, dom, st, b);
 #pragma unroll
         for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
@@ -429,7 +537,14 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
       cs_wait_all();  // and now holds the new ones
     }
   }
-  if (live) a.x.store(g, dom, st, xk);
+  if (!live) return;
+  a.x.store(g, dom, st, xk);
+  if (HALO && a.do_halo) {
+    cs_halo_out<0>(a, sl, D, jd, lc, s, xk);
+    cs_halo_out<1>(a, sl, D, jd, lc, s, xk);
+    cs_halo_out<2>(a, sl, D, jd, lc, s, xk);
+    if (lt == K - 1 || lt == 0) cs_halo_out<3>(a, sl, D, jd, lc, s, xk);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -507,7 +622,7 @@ static void cluster_staging(qcd_ctx* ctx, cudaStream_t st) {
 
 // M_SAP with one cluster per domain, nrhs stacked float32 fields
 void sap_cluster_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n_sap, int n_jac, void* ws_s,
-                       cudaStream_t st) {
+                       void* halo, cudaStream_t st) {
   cluster_staging(ctx, st);
   ClusterSapArgs a;
   a.g = ctx->geom;
@@ -519,6 +634,13 @@ void sap_cluster_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n
   }
   a.slice = a.sd[0] * a.sd[1] * a.sd[2];
   a.n_jac = n_jac;
+  a.halo = (float4*)halo;
+  size_t halo_f4 = 0;
+  for (int mu = 0; mu < 4; ++mu) {
+    a.face[mu] = a.slice * a.sd[3] / a.sd[mu];
+    a.halo_at[mu] = halo_f4;
+    halo_f4 += (size_t)3 * nsd * a.face[mu];
+  }
   a.kappa = (float)ctx->kappa;
   a.U16 = LinkPtrHalf{ctx->u16};
   a.links = (const unsigned char*)ctx->cl_link;
@@ -530,9 +652,13 @@ void sap_cluster_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n
   const int K = a.sd[3];
   const int threads = (a.slice + 31) / 32 * 32;
   const size_t smem = (size_t)CS_BYTES_PER_SITE * a.slice + CS_EXTRA_BYTES;
-  QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((size_t)CS_BYTES_PER_SITE * CS_MAX_SLICE + CS_EXTRA_BYTES)));
   const size_t v4 = (size_t)a.g.vol * 6;
+  // the caller's buffer holds 96 bytes per site; domains with several extents
+  // of one, whose faces need more, read the other colour's x in place
+  const bool with_halo = halo_f4 <= v4;
+  auto kernel = with_halo ? sap_cluster_kernel<true> : sap_cluster_kernel<false>;
+  QCD_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)((size_t)CS_BYTES_PER_SITE * CS_MAX_SLICE + CS_EXTRA_BYTES)));
   for (int r = 0; r < nrhs; ++r) {
     a.b = F32Spinor{(float4*)b + r * v4};
     a.x = F32Spinor{x + r * v4};
@@ -543,20 +669,25 @@ void sap_cluster_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n
       for (int colour = 0; colour < 2; ++colour) {
         a.colour = colour;
         a.do_surface = (sweep == 0 && colour == 0) ? 0 : 1;
+        a.do_halo = (sweep == n_sap && colour == 1) ? 0 : 1;
         LaunchScope ls(ctx, QCD_KC_SAP_BLOCK, st);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(nsd / 2 * K));
         cfg.blockDim = dim3(threads);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = K;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        QCD_CUDA_CHECK(cudaLaunchKernelEx(&cfg, sap_cluster_kernel, a));
+        // early start: not the first launch (what ran before may have built the
+        // staging copy), nor the kernel that reads x through L1
+        cfg.numAttrs = with_halo && (r > 0 || sweep > 0 || colour > 0) ? 2 : 1;
+        QCD_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, a));
         check_launch();
       }
     }

@@ -305,7 +305,7 @@ bool sap_domain_valid(const int dims[4], const int sdom[4]) {
 static const char* const kGeneralShapes[] = {"cluster_per_domain", "cta_per_domain"};
 
 void sap_general_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n_sap, int n_jac, int sap_prec,
-                       void* ws_s, cudaStream_t st) {
+                       void* ws_s, void* halo, cudaStream_t st) {
   QCD_REQUIRE(sap_prec == QCD_PREC_SINGLE || sap_prec == QCD_PREC_HALF_GAUGE, QCD_ERR_ARG,
               "SAP on general domains: sap_prec must be SINGLE or HALF_GAUGE");
   const bool can_cluster = sap_cluster_eligible(ctx, sap_prec);
@@ -317,7 +317,7 @@ void sap_general_apply(qcd_ctx* ctx, float4* x, const float4* b, int nrhs, int n
   const size_t v4 = (size_t)ctx->geom.vol * 6;
   auto run = [&](int v) {
     if (v == 0 && can_cluster) {
-      sap_cluster_apply(ctx, x, b, nrhs, n_sap, n_jac, ws_s, st);
+      sap_cluster_apply(ctx, x, b, nrhs, n_sap, n_jac, ws_s, halo, st);
       return;
     }
     for (int r = 0; r < nrhs; ++r) {
