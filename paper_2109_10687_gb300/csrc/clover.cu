@@ -10,9 +10,10 @@
 // (sigma_k (x) A = [[A_3, A_1 - i A_2], [A_1 + i A_2, -A_3]] on (spin, colour)),
 // each multiplied by i kappa c_SW.
 //
-// Two kernels: F of every site and plane (a thread each), then, a thread per
-// site and chiral block, 1 + C, its inverse in float64 and every copy of both
-// that the library keeps.  F waits in between in the buffer of 1 + C.
+// Two kernels: F of every site and plane (a thread each; in two shares, one
+// of which the neighbouring site's thread forms), then, a thread per site and
+// chiral block, 1 + C, its inverse in float64 and every copy of both that the
+// library keeps.
 //
 // What bounds them: this GPU has two float64 lanes per SM and cycle, and the
 // leaves and inverses in float64 (11.2 k fused multiply-adds per site, one
@@ -23,10 +24,11 @@
 // three 32x32 -> 64 multiply-adds (lo lo, below 2^-59 of one, is left out),
 // and a sum of products stays in 64 bits.  The error of a matrix product is
 // a few units of 2^-58 of the entries' bound, below float64's 2^-53.
-// On 24^3 x 48 F takes 2.8 ms (the multipliers busy 55 %; 3.0 ms with 168
-// registers and 12 warps, 3.2 ms with 96 and 20) and the inversion 1.36 ms
-// (the float64 pipe busy 84 %).  One kernel with a barrier between the two
-// took 5.4 ms.
+// On 24^3 x 48 F takes 1.62 ms (2.81 when a site formed its own four leaves,
+// in pairs, and not the staples it shares with its neighbours; 3.0 and 3.2 in
+// that form with 12 and 20 warps per SM instead of 16) and the inversion
+// 1.43 ms (the float64 pipe busy 84 %; it also adds the two shares of F).
+// One kernel with a barrier between the two took 5.4 ms in the older form.
 
 #include "fixed.cuh"
 #include "qcd_internal.cuh"
@@ -136,72 +138,84 @@ __device__ __forceinline__ FxMat fx_link(const Geom& g, const int4* __restrict__
   return m;
 }
 
-// F_mu,nu at x, as its nine independent reals: the imaginary parts of the
-// diagonal, then (re, im) of the entries 01, 02, 12.  Only Q - Q^dag is
-// needed, so a leaf may be replaced by minus its adjoint, and the four leaves
-// pair up by their first factor:
-//   Q - Q^dag = M - M^dag,  M = sum_h L (X - Y^dag)  over two halves h,
-// X and Y products of three links: ten matrix products instead of twelve.
-// Both halves and both triple products are loops over the same code, whose
-// instructions then fit the cache; X waits in shared memory (stash, this
-// thread's column of a [18][FS_THREADS] array) while Y is formed.
+// The link U_mu(x) belongs to two of x's leaves in the mu-nu plane and to two
+// of x + e_mu's, through the same two staples: with
+//   D = X - Y^dag,  X = U_nu(x+mu) U_mu^dag(x+nu) U_nu^dag(x),
+//                   Y = U_nu^dag(x-nu) U_mu(x-nu) U_nu(x+mu-nu),
+// Q - Q^dag of a site is [M - M^dag] over M = U_mu D at x and M = D U_mu at
+// x - e_mu.  So a thread forms the staples of one link and plane (four matrix
+// products) and both its M (one each, as U D and U^dag D^dag, whose
+// anti-Hermitian part is minus that of D U): six products per site and plane,
+// not the ten of a site's own leaves taken in pairs.  own and next get
+// 2^61 times the nine reals of this site's share and of x + e_mu's: the
+// imaginary parts of the diagonal, then (re, im) of the entries 01, 02, 12.
+// X and Y, and the two M, are loops over the same code, whose instructions
+// then fit the cache; X, then D, wait in shared memory (stash, this thread's
+// column of a [18][FS_THREADS] array).
 constexpr int FS_THREADS = 128;
 struct PathLink {  // direction (0 mu, 1 nu), offsets along mu and nu, adjoint
   signed char dir, dm, dn, dag;
 };
-// [half]: X's three links, Y's three, L
-__constant__ PathLink c_path[2][7] = {
-    {{1, 1, 0, 0}, {0, 0, 1, 1}, {1, 0, 0, 1}, {1, 0, -1, 1}, {0, 0, -1, 0}, {1, 1, -1, 0}, {0, 0, 0, 0}},
-    {{1, -1, -1, 1}, {0, -1, -1, 0}, {1, 0, -1, 0}, {1, 0, 0, 0}, {0, -1, 1, 1}, {1, -1, 0, 1}, {0, -1, 0, 1}},
-};
+__constant__ PathLink c_path[6] = {  // X's three links, Y's three
+    {1, 1, 0, 0}, {0, 0, 1, 1}, {1, 0, 0, 1}, {1, 0, -1, 1}, {0, 0, -1, 0}, {1, 1, -1, 0}};
+template <typename Store>
 __device__ __forceinline__ void field_strength_fx(const Geom& g, const int4* U, const int x[4], int mu, int nu,
-                                                  long long* stash, double f[9]) {
-  long long acc[9];
-#pragma unroll
-  for (int e = 0; e < 9; ++e) acc[e] = 0;
+                                                  long long* stash, const Store& store) {
+  auto link = [&](int k) {
+    const PathLink q = c_path[k];
+    return fx_link(g, U, x, mu, nu, q.dm, q.dn, q.dir ? nu : mu, q.dag != 0);
+  };
+  FxSum P;
+  FxMat t;
 #pragma unroll 1
-  for (int h = 0; h < 2; ++h) {
-    auto link = [&](int k) {
-      const PathLink q = c_path[h][k];
-      return fx_link(g, U, x, mu, nu, q.dm, q.dn, q.dir ? nu : mu, q.dag != 0);
-    };
-    FxSum P;
-    FxMat t;
-#pragma unroll 1
-    for (int q = 0; q < 2; ++q) {
-      fx_mul(link(3 * q), link(3 * q + 1), P);
-      fx_limbs(P, t);
-      fx_mul(t, link(3 * q + 2), P);
-      if (q == 0) {
+  for (int q = 0; q < 2; ++q) {
+    fx_mul(link(3 * q), link(3 * q + 1), P);
+    fx_limbs(P, t);
+    fx_mul(t, link(3 * q + 2), P);
 #pragma unroll
-        for (int e = 0; e < 9; ++e) {
-          stash[2 * e * FS_THREADS] = P.re[e / 3][e % 3];
-          stash[(2 * e + 1) * FS_THREADS] = P.im[e / 3][e % 3];
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        long long *re = stash + 2 * (3 * i + j) * FS_THREADS, *im = re + FS_THREADS;
+        if (q == 0) {
+          *re = P.re[i][j];
+          *im = P.im[i][j];
+        } else {  // D = X - Y^dag
+          *re -= P.re[j][i];
+          *im += P.im[j][i];
         }
       }
-    }
-    FxSum D;  // X - Y^dag
+  }
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    // U D, then U^dag D^dag
+    const int row = h ? 1 : 3, col = h ? 3 : 1;
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      D.re[e / 3][e % 3] = stash[2 * e * FS_THREADS] - P.re[e % 3][e / 3];
-      D.im[e / 3][e % 3] = stash[(2 * e + 1) * FS_THREADS] + P.im[e % 3][e / 3];
-    }
-    fx_limbs(D, t);
-    fx_mul(link(6), t, P);
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int i = 0; i < 3; ++i) acc[i] += 2 * P.im[i][i];
+      for (int j = 0; j < 3; ++j) {
+        const long long* d = stash + 2 * (row * i + col * j) * FS_THREADS;
+        P.re[i][j] = d[0];
+        P.im[i][j] = h ? -d[FS_THREADS] : d[FS_THREADS];
+      }
+    fx_limbs(P, t);
+    fx_mul(fx_link(g, U, x, mu, nu, 0, 0, mu, h != 0), t, P);
+    long long f[9];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) f[i] = 2 * P.im[i][i];
     int o = 3;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int j = i + 1; j < 3; ++j) {
-        acc[o++] += P.re[i][j] - P.re[j][i];
-        acc[o++] += P.im[i][j] + P.im[j][i];
+        f[o++] = P.re[i][j] - P.re[j][i];
+        f[o++] = P.im[i][j] + P.im[j][i];
       }
-  }
-  const double u = 1.0 / (double)(1LL << FX_FRAC) / 8.0;  // a power of two
+    if (h)
 #pragma unroll
-  for (int e = 0; e < 9; ++e) f[e] = u * (double)acc[e];
+      for (int e = 0; e < 9; ++e) f[e] = -f[e];
+    store(h, f);
+  }
 }
 
 // inverse by Gauss-Jordan with partial pivoting, for blocks that are not
@@ -316,19 +330,10 @@ __device__ __noinline__ bool invert6_general(double* r, int stride) {
   return ok;
 }
 
-// chiral block b of 1 + C from the six F (nine reals each, read by f(plane, e)):
+// a chiral block of 1 + C from kc A_1, kc A_2, kc A_3 (nine reals each):
 // 1 + [[H_3, H_1 - i H_2], [H_1 + i H_2, -H_3]], H_k = i kc A_k Hermitian
-template <typename F>
-__device__ __forceinline__ void pack_block(const F& f, int b, double kc, double m[36]) {
-  // planes 0 xy, 1 xz, 2 xt, 3 yz, 4 yt, 5 zt
-  const double sg = b == 0 ? 1.0 : -1.0;
-  double a1[9], a2[9], a3[9];
-#pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    a1[e] = kc * fma(sg, f(2, e), -f(3, e));
-    a2[e] = kc * fma(sg, f(4, e), f(1, e));
-    a3[e] = kc * fma(sg, f(5, e), -f(0, e));
-  }
+__device__ __forceinline__ void pack_block(const double a1[9], const double a2[9], const double a3[9],
+                                           double m[36]) {
   // entry (i, j) of i A for A given as the nine reals
   auto h = [](const double a[9], int i, int j) {
     if (i == j) return make_cx(-a[i], 0.0);
@@ -370,10 +375,13 @@ struct CloverOut {
   float4* st32;               // [dom][site][19]
 };
 
-// F between the kernels: a plane's nine reals in five double2 (the last half
-// filled), component 5 plane + k of [dom][36][vd] -- each site's own entries
-// of the buffer that 1 + C overwrites
+// F between the kernels: a plane's nine reals in five pairs (the last half
+// filled), pair 5 plane + k of [dom][36][vd]: float64 in the buffer of 1 + C
+// (each site's own entries, which 1 + C overwrites), or fixed point, the
+// site's own share there and the next site's in a second buffer
 constexpr int F_PAIRS = 5;
+__host__ __device__ constexpr int plane_mu(int p) { return p < 3 ? 0 : (p < 5 ? 1 : 2); }
+__host__ __device__ constexpr int plane_nu(int p) { return p < 3 ? p + 1 : (p < 5 ? p - 1 : 3); }
 
 // A warp takes 32 consecutive sites (in lexicographic-domain order, so that
 // neighbouring domains' links are still in L2) and one plane; the six planes
@@ -383,7 +391,8 @@ constexpr int F_PAIRS = 5;
 // two thirds idle).
 template <bool FIXED>
 __global__ void __launch_bounds__(FS_THREADS, 4) field_strength_kernel(Geom g, const int4* __restrict__ ufx,
-                                                                       LinkPtr<double> U, double2* out) {
+                                                                       LinkPtr<double> U, double2* out,
+                                                                       longlong2* next) {
   __shared__ long long stash[FIXED ? 18 * FS_THREADS : 1];
   const int lane = threadIdx.x & 31;
   const long long item = blockIdx.x * (long long)(FS_THREADS / 32) + (threadIdx.x >> 5);
@@ -399,20 +408,44 @@ __global__ void __launch_bounds__(FS_THREADS, 4) field_strength_kernel(Geom g, c
     x[mu] = (lex - q * g.nd[mu]) * g.d[mu] + ((s >> g.shift[mu]) & (g.d[mu] - 1));
     lex = q;
   }
-  const int mu = p < 3 ? 0 : (p < 5 ? 1 : 2);
-  const int nu = p < 3 ? p + 1 : (p < 5 ? p - 1 : 3);
-  double f[10];
-  f[9] = 0.0;
-  if (FIXED) field_strength_fx(g, ufx, x, mu, nu, stash + threadIdx.x, f);
-  else field_strength(g, U, x, mu, nu, f);
+  const int mu = plane_mu(p), nu = plane_nu(p);
+  const size_t at = (((size_t)(dom * 36 + F_PAIRS * p)) << g.logvd) + s;
+  if (FIXED) {
+    field_strength_fx(g, ufx, x, mu, nu, stash + threadIdx.x, [&](int h, const long long f[9]) {
+      longlong2* q = (h ? next : reinterpret_cast<longlong2*>(out)) + at;
 #pragma unroll
-  for (int k = 0; k < F_PAIRS; ++k)
-    out[(((size_t)(dom * 36 + F_PAIRS * p + k)) << g.logvd) + s] = make_double2(f[2 * k], f[2 * k + 1]);
+      for (int k = 0; k < F_PAIRS; ++k) q[(size_t)k << g.logvd] = make_longlong2(f[2 * k], k < 4 ? f[2 * k + 1] : 0);
+    });
+  } else {
+    double f[10];
+    f[9] = 0.0;
+    field_strength(g, U, x, mu, nu, f);
+#pragma unroll
+    for (int k = 0; k < F_PAIRS; ++k) out[at + ((size_t)k << g.logvd)] = make_double2(f[2 * k], f[2 * k + 1]);
+  }
 }
 
 // float64 rounded to float32 on the bit fields (conversions would queue on
 // the float64 pipe; results below float32's normal range become zero)
 __device__ __forceinline__ float to_float(double d) { return df64_from_double_scaled(d, 0).hi; }
+
+// F of a plane at a site, fixed point: the site's own share and the one that
+// the thread of the site before it along mu left
+__device__ __forceinline__ void fx_plane(const Geom& g, const double2* own, const longlong2* __restrict__ next, int dom,
+                                         int s, int p, long long f[10]) {
+  const int mu = plane_mu(p), step = 1 << g.shift[mu];
+  const bool inside = ((s >> g.shift[mu]) & (g.d[mu] - 1)) > 0;
+  const int bd = inside ? dom : __ldg(g.nbr + dom * 8 + 2 * mu + 1);
+  const int bs = inside ? s - step : s + (g.d[mu] - 1) * step;
+  const longlong2* u = reinterpret_cast<const longlong2*>(own) + (((size_t)(dom * 36 + F_PAIRS * p)) << g.logvd) + s;
+  const longlong2* v = next + (((size_t)(bd * 36 + F_PAIRS * p)) << g.logvd) + bs;
+#pragma unroll
+  for (int k = 0; k < F_PAIRS; ++k) {
+    const longlong2 a = u[(size_t)k << g.logvd], b = __ldg(v + ((size_t)k << g.logvd));
+    f[2 * k] = a.x + b.x;
+    f[2 * k + 1] = a.y + b.y;
+  }
+}
 
 // Threads (site, block): warps 0 and 1 the two blocks of 32 sites, warps 2
 // and 3 those of the next 32.  The float64 pipe bounds it (the inversion);
@@ -421,7 +454,9 @@ __device__ __forceinline__ float to_float(double d) { return df64_from_double_sc
 constexpr int CB_THREADS = 128;
 constexpr int CB_SITES = CB_THREADS / 2;
 constexpr int CB_ROW = 73;  // floats per site in shared memory, odd: no bank conflicts
-__global__ void __launch_bounds__(CB_THREADS, 4) clover_build_kernel(Geom g, double kc, CloverOut o, int* status) {
+template <bool FIXED>
+__global__ void __launch_bounds__(CB_THREADS, 4) clover_build_kernel(Geom g, double kc, CloverOut o,
+                                                                     const longlong2* __restrict__ next, int* status) {
   __shared__ float stage[CB_SITES * CB_ROW];
   __shared__ double rows[36 * CB_THREADS];  // the pivoted inversion's operand and result
   const int b = (threadIdx.x >> 5) & 1;
@@ -433,14 +468,37 @@ __global__ void __launch_bounds__(CB_THREADS, 4) clover_build_kernel(Geom g, dou
   const size_t at = ((size_t)dom * 36 << g.logvd) + s;
   double m[36];
   {
-    double f[60];
+    // A_k = +- F_p + or - F_q, planes 0 xy, 1 xz, 2 xt, 3 yz, 4 yt, 5 zt; the
+    // upper sign of F_p in block 0
+    constexpr int P[3] = {2, 4, 5}, Q[3] = {3, 1, 0};
+    double a[3][9];
 #pragma unroll
-    for (int k = 0; k < 6 * F_PAIRS; ++k) {
-      const double2 v = o.clov64[at + ((size_t)k << g.logvd)];
-      f[2 * k] = v.x;
-      f[2 * k + 1] = v.y;
+    for (int k = 0; k < 3; ++k) {
+      if (FIXED) {
+        // exact sums of 62 bits at most, converted once; 2^-61 comes with kc
+        long long f[10], h[10];
+        fx_plane(g, o.clov64, next, dom, s, P[k], f);
+        fx_plane(g, o.clov64, next, dom, s, Q[k], h);
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+          const long long v = b == 0 ? f[e] : -f[e];
+          a[k][e] = kc * (double)(k == 1 ? v + h[e] : v - h[e]);
+        }
+      } else {
+        const double sg = b == 0 ? 1.0 : -1.0;
+        double f[10], h[10];
+#pragma unroll
+        for (int i = 0; i < F_PAIRS; ++i) {
+          const double2 u = o.clov64[at + ((size_t)(F_PAIRS * P[k] + i) << g.logvd)];
+          const double2 v = o.clov64[at + ((size_t)(F_PAIRS * Q[k] + i) << g.logvd)];
+          f[2 * i] = u.x; f[2 * i + 1] = u.y;
+          h[2 * i] = v.x; h[2 * i + 1] = v.y;
+        }
+#pragma unroll
+        for (int e = 0; e < 9; ++e) a[k][e] = kc * fma(sg, f[e], k == 1 ? h[e] : -h[e]);
+      }
     }
-    pack_block([&](int p, int e) { return f[2 * F_PAIRS * p + e]; }, b, kc, m);
+    pack_block(a[0], a[1], a[2], m);
   }
   __syncthreads();  // every F of the block is read before 1 + C overwrites it
   if (live) {
@@ -521,25 +579,25 @@ void build_clover_launch(qcd_ctx* ctx, cudaStream_t st) {
                     (uint4*)ctx->st_clov16, (float4*)ctx->st_clov32};
   const int grid = grid_for((g.vol + 31) / 32 * 6, FS_THREADS / 32);
   const LinkPtr<double> U{ctx->u64};
+  const double kc = ctx->kappa * ctx->csw;
+  const int sites = grid_for(g.vol, CB_SITES);
+  auto launch = [&](auto kernel, int blocks, int threads, auto... args) {
+    LaunchScope ls(ctx, QCD_KC_OTHER, st);
+    kernel<<<blocks, threads, 0, st>>>(args...);
+    check_launch();
+  };
   if (ctx->su3_links) {
-    // the limbs lie where the double-float links go once the clover term is built
-    int4* ufx = reinterpret_cast<int4*>(ctx->udf);
-    {
-      LaunchScope ls(ctx, QCD_KC_OTHER, st);
-      links_to_fixed_kernel<<<1216, 256, 0, st>>>(ctx->u64, ufx, (size_t)g.vol * 36);
-      check_launch();
-    }
-    LaunchScope ls(ctx, QCD_KC_OTHER, st);
-    field_strength_kernel<true><<<grid, FS_THREADS, 0, st>>>(g, ufx, U, ctx->clov64);
-    check_launch();
+    // scratch: the limbs where 1 + C goes in double-float, the next sites'
+    // shares of F where the double-float links go once the clover term is built
+    int4* ufx = reinterpret_cast<int4*>(ctx->clovdf);
+    longlong2* next = reinterpret_cast<longlong2*>(ctx->udf);
+    launch(links_to_fixed_kernel, 1216, 256, ctx->u64, ufx, (size_t)g.vol * 36);
+    launch(field_strength_kernel<true>, grid, FS_THREADS, g, ufx, U, ctx->clov64, next);
+    launch(clover_build_kernel<true>, sites, CB_THREADS, g, kc / (double)(8LL << FX_FRAC), o, next, ctx->d_status);
   } else {
-    LaunchScope ls(ctx, QCD_KC_OTHER, st);
-    field_strength_kernel<false><<<grid, FS_THREADS, 0, st>>>(g, nullptr, U, ctx->clov64);
-    check_launch();
+    launch(field_strength_kernel<false>, grid, FS_THREADS, g, nullptr, U, ctx->clov64, nullptr);
+    launch(clover_build_kernel<false>, sites, CB_THREADS, g, kc, o, nullptr, ctx->d_status);
   }
-  LaunchScope ls(ctx, QCD_KC_OTHER, st);
-  clover_build_kernel<<<grid_for(g.vol, CB_SITES), CB_THREADS, 0, st>>>(g, ctx->kappa * ctx->csw, o, ctx->d_status);
-  check_launch();
 }
 
 }  // namespace qcd

@@ -798,7 +798,7 @@ void clover_apply_launch(qcd_ctx* ctx, void* out, const void* in, int prec, int 
                          cudaStream_t st);
 void ablock_launch(qcd_ctx* ctx, float4* out, const float4* in, int row, int col, cudaStream_t st);
 // build_clover_launch writes every copy of 1 + C and its inverse and uses
-// ctx->udf as scratch; build_link_copies then writes the double-float links
+// ctx->udf and ctx->clovdf as scratch; build_link_copies then writes the double-float links
 // there and the staged links of the SAP block kernel
 void build_clover_launch(qcd_ctx* ctx, cudaStream_t st);
 void build_link_copies(qcd_ctx* ctx, cudaStream_t st);
