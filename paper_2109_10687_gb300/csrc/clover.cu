@@ -24,9 +24,9 @@
 // three 32x32 -> 64 multiply-adds (lo lo, below 2^-59 of one, is left out),
 // and a sum of products stays in 64 bits.  The error of a matrix product is
 // a few units of 2^-58 of the entries' bound, below float64's 2^-53.
-// On 24^3 x 48 F takes 1.62 ms (2.81 when a site formed its own four leaves,
-// in pairs, and not the staples it shares with its neighbours; 3.0 and 3.2 in
-// that form with 12 and 20 warps per SM instead of 16) and the inversion
+// On 24^3 x 48 F takes 1.56 ms with 12 warps per SM (1.62 with 16, 1.78 with
+// 20; 2.81 when a site formed its own four leaves, in pairs, and not the
+// staples it shares with its neighbours) and the inversion
 // 1.43 ms (the float64 pipe busy 84 %; it also adds the two shares of F).
 // One kernel with a barrier between the two took 5.4 ms in the older form.
 
@@ -386,11 +386,10 @@ __host__ __device__ constexpr int plane_nu(int p) { return p < 3 ? p + 1 : (p < 
 // A warp takes 32 consecutive sites (in lexicographic-domain order, so that
 // neighbouring domains' links are still in L2) and one plane; the six planes
 // of a tile are consecutive warps and share its links through L1.  No
-// barrier and 128 registers: 16 warps per SM keep the multipliers busy
-// (phases of one fused kernel, with 12 warps and its barriers, left them
-// two thirds idle).
+// barrier, so that the warps' loads and products overlap (phases of one fused
+// kernel, with its barriers, left the multipliers two thirds idle).
 template <bool FIXED>
-__global__ void __launch_bounds__(FS_THREADS, 4) field_strength_kernel(Geom g, const int4* __restrict__ ufx,
+__global__ void __launch_bounds__(FS_THREADS, 3) field_strength_kernel(Geom g, const int4* __restrict__ ufx,
                                                                        LinkPtr<double> U, double2* out,
                                                                        longlong2* next) {
   __shared__ long long stash[FIXED ? 18 * FS_THREADS : 1];

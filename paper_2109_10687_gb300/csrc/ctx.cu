@@ -277,14 +277,17 @@ __device__ __forceinline__ double su3_deviation_fx(const double* in, unsigned lo
 // canonical gauge field -> internal float64 / float32 / float16 links and
 // float32 two-row links, with an SU(3) check that records the worst deviation
 // in bad[0] (as the bit pattern of a non-negative double, so integer atomicMax
-// orders it; NaN entries drop out of it) and any non-finite entry in bad[1].  A block takes 64 sites in internal order, a thread one link:
-// the canonical reads (576 contiguous bytes a site) go through shared memory,
-// and every write is one stream over consecutive sites.  24^3 x 48: 0.62 ms;
-// one thread per site reading its 72 doubles itself, check in float64, 0.88 ms.
-constexpr int GI_SITES = 64;
+// orders it; NaN entries drop out of it) and any non-finite entry in bad[1].
+// A block takes 32 sites in internal order, a thread one link: the canonical
+// reads (576 contiguous bytes a site) go through shared memory, and every
+// write is one stream over consecutive sites.  Latency bounds it (loads,
+// barrier, arithmetic, stores), so small blocks, many per SM: 24^3 x 48
+// 0.50 ms; 64 sites a block 0.64 (two blocks per SM), 0.52 (three); one thread
+// per site reading its 72 doubles itself, check in float64, 0.88 ms.
+constexpr int GI_SITES = 32;
 constexpr int GI_THREADS = 4 * GI_SITES;
 constexpr int GI_ROW = 73;  // doubles per site in shared memory
-__global__ void __launch_bounds__(GI_THREADS, 2) gauge_import_kernel(Geom g, const double* __restrict__ src,
+__global__ void __launch_bounds__(GI_THREADS, 6) gauge_import_kernel(Geom g, const double* __restrict__ src,
                                                                   double2* u64, float2* u32, __half2* u16,
                                                                   float4* u32c, unsigned long long* bad) {
   __shared__ double buf[GI_SITES * GI_ROW];
