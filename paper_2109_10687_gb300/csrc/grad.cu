@@ -13,7 +13,8 @@
 //            R_k = A_{k+1} .. A_4 V_p(n) A_1 .. A_{k-1} (R_k^dag for an
 //            undaggered factor).
 // The clover part is gathered per link (no atomics): each thread owns one
-// link U_d(y) and visits the 24 (plane, leaf, factor) slots where it occurs.
+// link U_d(y), which lies on six plaquettes, each of them a leaf of the Q of
+// its four corners.
 
 #include "qcd_internal.cuh"
 
@@ -33,6 +34,15 @@ __device__ __forceinline__ void mm(const M3f& a, const M3f& b, M3f& c) {
       c.m[i][j] = acc;
     }
 }
+// c += a b
+__device__ __forceinline__ void mma(const M3f& a, const M3f& b, M3f& c) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) c.m[i][j] = cmac(c.m[i][j], a.m[i][k], b.m[k][j]);
+}
 __device__ __forceinline__ M3f dg(const M3f& a) {
   M3f r;
 #pragma unroll
@@ -46,26 +56,6 @@ __device__ __forceinline__ void coords_of(const Geom& g, long long n, int x[4]) 
 
 // periodic wrap of a coordinate at most one period outside [0, L)
 __device__ __forceinline__ int wrap1(int v, int L) { return v < 0 ? v + L : (v >= L ? v - L : v); }
-
-// internal (domain, site) of x + off, |off_k| <= 1
-__device__ __forceinline__ void at_coords(const Geom& g, const int x[4], const int off[4], int& dom, int& s) {
-  int y[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) y[k] = wrap1(x[k] + off[k], g.L[k]);
-  coords_to_internal(g, y, dom, s);
-}
-
-// leaves of Q_{mu nu}(n): (direction: 0 = mu, 1 = nu; offset along mu; offset
-// along nu; daggered)
-struct LeafFactor {
-  signed char dir, om, on, dag;
-};
-__constant__ LeafFactor c_leaf[4][4] = {
-    {{0, 0, 0, 0}, {1, 1, 0, 0}, {0, 0, 1, 1}, {1, 0, 0, 1}},
-    {{1, 0, 0, 0}, {0, -1, 1, 1}, {1, -1, 0, 1}, {0, -1, 0, 0}},
-    {{0, -1, 0, 1}, {1, -1, -1, 1}, {0, -1, -1, 0}, {1, 0, -1, 0}},
-    {{1, 0, -1, 1}, {0, 0, -1, 0}, {1, 1, -1, 0}, {0, 0, 0, 1}},
-};
 
 // plane index of (mu < nu): 0 xy, 1 xz, 2 xt, 3 yz, 4 yt, 5 zt
 __host__ __device__ __forceinline__ int plane_index(int mu, int nu) {
@@ -183,7 +173,12 @@ __device__ void hop_force(const Geom& g, const F32Spinor& xs, const F32Spinor& l
 }
 
 // one thread per link (y, d): G = G_hop + G_clover; project: TA(G U^dag)
-__global__ void __launch_bounds__(128) force_kernel(Geom g, F32Spinor xs, F32Spinor ls, LinkPtr<float> U,
+// The clover part, bound by its 3x3 products and gathers: eight products and
+// seven matrices loaded per plaquette, which serve the leaves of all four
+// corners.  16^4: 0.155 ms (12 warps per SM; 8 and 16 0.162 and 0.160); with
+// each of the 24 (plane, leaf, factor) slots by itself, four products and four
+// matrices each, 0.313 ms.
+__global__ void __launch_bounds__(128, 3) force_kernel(Geom g, F32Spinor xs, F32Spinor ls, LinkPtr<float> U,
                                                     const float2* V, float kappa, int with_clover, int project,
                                                     double* out) {
   // a block takes 32 sites, warp d their links in direction d: the
@@ -206,56 +201,63 @@ __global__ void __launch_bounds__(128) force_kernel(Geom g, F32Spinor xs, F32Spi
     default: hop_force<3>(g, xs, ls, dom, s, kappa, G); break;
   }
   if (with_clover) {
-    for (int other = 0; other < 4; ++other) {
-      if (other == d) continue;
-      const int mu = d < other ? d : other, nu = d < other ? other : d;
-      const int p = plane_index(mu, nu);
-      const int my_dir = d == mu ? 0 : 1;
-      for (int leaf = 0; leaf < 4; ++leaf)
-        for (int k = 0; k < 4; ++k) {
-          const LeafFactor fk = c_leaf[leaf][k];
-          if (fk.dir != my_dir) continue;
-          // site n of the leaf: y = n + offset_k
-          int base[4] = {0, 0, 0, 0};
-          base[mu] -= fk.om;
-          base[nu] -= fk.on;
-          int xn[4];
+#pragma unroll 1
+    for (int k = 0; k < 6; ++k) {
+      const int e = k >> 1 < d ? k >> 1 : (k >> 1) + 1;  // the plaquette's other direction
+      const int side = k & 1 ? -1 : 1;
+      const bool dag = (d < e) == (side < 0);  // the loop runs against U_d(y)
+      const int p = plane_index(min(d, e), max(d, e));
+      // from the end of U_d(y) (or of its adjoint) around to its start: C1
+      // along side * e, C2 against (or along) d, C3 back; the loop's corners
+      // after each factor are a, b, c, and d after C3
+      const int a1 = dag ? 0 : 1;
+      auto point = [&](int od, int oe, int x[4]) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) xn[q] = wrap1(y[q] + base[q], g.L[q]);
-          const long long nn = canon_index(g, xn);
-          // R_k = A_{k+1} .. A_4 V A_1 .. A_{k-1}
-          M3f r;
-          for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j) r.m[i][j] = make_cx(i == j ? 1.f : 0.f, 0.f);
-          auto factor = [&](int j) {
-            const LeafFactor f = c_leaf[leaf][j];
-            int off[4] = {0, 0, 0, 0};
-            off[mu] += f.om;
-            off[nu] += f.on;
-            int fd, fs;
-            at_coords(g, xn, off, fd, fs);
-            M3f u;
-            U.load(g, fd, f.dir == 0 ? mu : nu, fs, u);
-            return f.dag ? dg(u) : u;
-          };
-          M3f tmp;
-          for (int j = k + 1; j < 4; ++j) {
-            const M3f a = factor(j);
-            mm(r, a, tmp);
-            r = tmp;
+        for (int q = 0; q < 4; ++q) x[q] = wrap1(y[q] + (q == d ? od : 0) + (q == e ? oe : 0), g.L[q]);
+      };
+      auto link = [&](int dir, int od, int oe, bool adj) {
+        int x[4], fd, fs;
+        point(od, oe, x);
+        coords_to_internal(g, x, fd, fs);
+        const float2* q = U.p + (((size_t)((fd * 4 + dir) * 9)) << g.logvd) + fs;
+        const int row = adj ? 1 : 3, col = adj ? 3 : 1;
+        M3f u;
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float2 v = __ldg(q + ((size_t)(r * row + c * col) << g.logvd));
+            u.m[r][c] = make_cx(v.x, adj ? -v.y : v.y);
           }
-          const M3f v = load_v(g, V, p, nn);
-          mm(r, v, tmp);
-          r = tmp;
-          for (int j = 0; j < k; ++j) {
-            const M3f a = factor(j);
-            mm(r, a, tmp);
-            r = tmp;
-          }
-          const M3f c = fk.dag ? r : dg(r);
-          for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j) G.m[i][j] = G.m[i][j] + c.m[i][j];
-        }
+        return u;
+      };
+      auto corner = [&](int od, int oe) {
+        int x[4];
+        point(od, oe, x);
+        return load_v(g, V, p, canon_index(g, x));
+      };
+      const int oe = side < 0 ? -1 : 0;
+      // R = V_a C1 C2 C3 + C1 V_b C2 C3 + C1 C2 V_c C3 + C1 C2 C3 V_d
+      M3f sum, t, c = link(e, a1, oe, side < 0);
+      mm(corner(a1, 0), c, sum);
+      mma(c, corner(a1, side), sum);
+      {
+        const M3f c2 = link(d, 0, side, !dag);
+        mm(c, c2, t);
+        mm(sum, c2, c);
+      }
+      mma(t, corner(1 - a1, side), c);
+      {
+        const M3f c3 = link(e, 1 - a1, oe, side > 0);
+        mm(c, c3, sum);
+        mm(t, c3, c);
+      }
+      mma(c, corner(1 - a1, 0), sum);
+      const M3f r = dag ? sum : dg(sum);
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) G.m[i][j] = G.m[i][j] + r.m[i][j];
     }
   }
   if (project) {
