@@ -113,12 +113,10 @@ constexpr int CONV_THREADS = 128;
 constexpr int CONV_STRIDE = 25;
 
 template <int PREC>
-__global__ void __launch_bounds__(CONV_THREADS) import_spinor_kernel(Geom g, void* dst, const double* __restrict__ src,
-                                                                     int nrhs, int paper_basis) {
+__device__ __forceinline__ void import_sites(const Geom& g, void* dst, const double* __restrict__ src, int rhs,
+                                             int nrhs, int paper_basis, long long n0) {
   __shared__ double buf[CONV_THREADS * CONV_STRIDE];
-  const long long n0 = blockIdx.x * (long long)CONV_THREADS;
   const long long n = n0 + threadIdx.x;
-  const int rhs = blockIdx.y;
   const int nsites = (int)min((long long)CONV_THREADS, g.vol - n0);
   const double* in = src + ((size_t)rhs * g.vol + n0) * 24;
   for (int i = threadIdx.x; i < nsites * 24; i += CONV_THREADS) buf[(i / 24) * CONV_STRIDE + i % 24] = in[i];
@@ -158,12 +156,16 @@ __global__ void __launch_bounds__(CONV_THREADS) import_spinor_kernel(Geom g, voi
 }
 
 template <int PREC>
-__global__ void __launch_bounds__(CONV_THREADS) export_spinor_kernel(Geom g, double* __restrict__ dst, const void* src,
+__global__ void __launch_bounds__(CONV_THREADS) import_spinor_kernel(Geom g, void* dst, const double* __restrict__ src,
                                                                      int nrhs, int paper_basis) {
+  import_sites<PREC>(g, dst, src, blockIdx.y, nrhs, paper_basis, blockIdx.x * (long long)CONV_THREADS);
+}
+
+template <int PREC>
+__device__ __forceinline__ void export_sites(const Geom& g, double* __restrict__ dst, const void* src, int rhs,
+                                             int nrhs, int paper_basis, long long n0) {
   __shared__ double buf[CONV_THREADS * CONV_STRIDE];
-  const long long n0 = blockIdx.x * (long long)CONV_THREADS;
   const long long n = n0 + threadIdx.x;
-  const int rhs = blockIdx.y;
   const int nsites = (int)min((long long)CONV_THREADS, g.vol - n0);
   if (n < g.vol) {
     int x[4];
@@ -204,6 +206,42 @@ __global__ void __launch_bounds__(CONV_THREADS) export_spinor_kernel(Geom g, dou
   __syncthreads();
   double* out = dst + ((size_t)rhs * g.vol + n0) * 24;
   for (int i = threadIdx.x; i < nsites * 24; i += CONV_THREADS) out[i] = buf[(i / 24) * CONV_STRIDE + i % 24];
+}
+template <int PREC>
+__global__ void __launch_bounds__(CONV_THREADS) export_spinor_kernel(Geom g, double* __restrict__ dst, const void* src,
+                                                                     int nrhs, int paper_basis) {
+  export_sites<PREC>(g, dst, src, blockIdx.y, nrhs, paper_basis, blockIdx.x * (long long)CONV_THREADS);
+}
+
+// Ragged batch: the float64 fields of every lattice in one launch, a block of
+// 128 sites by the block-to-lattice table.  Memory bounds it; a launch per
+// lattice left most of the GPU idle: 32 lattices with extents 8 and 16 (524 k
+// sites), import 166 -> 72 us, export 146 -> 52 us.
+__global__ void __launch_bounds__(CONV_THREADS) lat_import_kernel(const LatDesc* __restrict__ desc,
+                                                                  const int* __restrict__ block_lat,
+                                                                  const LatField* __restrict__ field, int to_b) {
+  const int lat = __ldg(block_lat + blockIdx.x);
+  const LatDesc& d = desc[lat];
+  import_sites<QCD_PREC_DOUBLE>(d.g, to_b ? d.b64 : d.x64, field[lat].p, 0, 1, field[lat].paper_basis,
+                                (blockIdx.x - d.block_begin) * CONV_THREADS);
+}
+__global__ void __launch_bounds__(CONV_THREADS) lat_export_kernel(const LatDesc* __restrict__ desc,
+                                                                  const int* __restrict__ block_lat,
+                                                                  const LatField* __restrict__ field) {
+  const int lat = __ldg(block_lat + blockIdx.x);
+  const LatDesc& d = desc[lat];
+  export_sites<QCD_PREC_DOUBLE>(d.g, field[lat].p, d.x64, 0, 1, field[lat].paper_basis,
+                                (blockIdx.x - d.block_begin) * CONV_THREADS);
+}
+void lat_import_launch(const LatDesc* d_lat, const int* d_block_lat, long long blocks, const LatField* d_field,
+                       bool to_b, cudaStream_t st) {
+  lat_import_kernel<<<(unsigned)blocks, CONV_THREADS, 0, st>>>(d_lat, d_block_lat, d_field, to_b);
+  check_launch();
+}
+void lat_export_launch(const LatDesc* d_lat, const int* d_block_lat, long long blocks, const LatField* d_field,
+                       cudaStream_t st) {
+  lat_export_kernel<<<(unsigned)blocks, CONV_THREADS, 0, st>>>(d_lat, d_block_lat, d_field);
+  check_launch();
 }
 
 // max over the entries of |Re| + |Im| of U^dag U - 1, and of det U - 1

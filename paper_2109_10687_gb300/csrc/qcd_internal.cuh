@@ -890,6 +890,17 @@ void lat_dslash_launch(const LatDesc* d_lat, const int* d_block_lat, long long b
 void lat_dslash_df64_launch(const LatDesc* d_lat, const int* d_tile_lat, long long tiles, const double* d_b2,
                             cudaStream_t st);
 
+// A lattice's canonical float64 field in a batch: the device copy of the
+// caller's pointers.  x64 or b64 of every lattice from them, x64 to them.
+struct LatField {
+  double* p;
+  int paper_basis;
+};
+void lat_import_launch(const LatDesc* d_lat, const int* d_block_lat, long long blocks, const LatField* d_field,
+                       bool to_b, cudaStream_t st);
+void lat_export_launch(const LatDesc* d_lat, const int* d_block_lat, long long blocks, const LatField* d_field,
+                       cudaStream_t st);
+
 // M_SAP (Algorithm 1) of every lattice of a ragged batch in shared launches:
 // one launch per half-sweep covers every lattice's domains of that colour.
 struct SapLat {

@@ -48,6 +48,8 @@ struct RaggedWS {
   int* h_ctrl = nullptr;   // pinned
   double* dres = nullptr;  // [0, n) |b|^2, [n, 2n) |r|^2, [2n, 3n) per-lattice scale
   double* h_res = nullptr; // pinned copy
+  LatField* d_field = nullptr;  // the caller's b of every lattice, then its x (on_device)
+  LatField* h_field = nullptr;  // pinned
   int* d_status = nullptr; // QCD_ERR_TIMEOUT from a bounded wait in a SAP launch
   int nblocks = 0;
   LatDesc* d_lat = nullptr;
@@ -69,12 +71,14 @@ void ragged_free(RaggedWS* w) {
   if (!w) return;
   void* ptrs[] = {w->d_v4off, w->d_v4len, w->d_n2off, w->d_n2len, w->x, w->r, w->p, w->q, w->t, w->zp, w->zr,
                   w->rt, w->b32, w->sap_s, w->halo, w->x64, w->r64, w->b64, w->partials, w->counters, w->scal,
-                  w->ctrl, w->dres, w->d_status, w->d_lat, w->d_site_lat, w->xdf, w->d_tile_lat};
+                  w->ctrl, w->dres, w->d_status, w->d_lat, w->d_site_lat, w->xdf, w->d_tile_lat,
+                  w->d_field};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (w->h_scal) cudaFreeHost(w->h_scal);
   if (w->h_ctrl) cudaFreeHost(w->h_ctrl);
   if (w->h_res) cudaFreeHost(w->h_res);
+  if (w->h_field) cudaFreeHost(w->h_field);
   sap_batch_free(w->plan_p);
   sap_batch_free(w->plan_r);
   if (w->loop) cudaGraphExecDestroy(w->loop);
@@ -266,6 +270,8 @@ static RaggedWS* ragged_ws(const std::vector<qcd_ctx*>& ctx, RaggedWS*& wp) {
     QCD_CUDA_CHECK(cudaMallocHost(&w->h_ctrl, sizeof(int) * 4));
     QCD_CUDA_CHECK(cudaMalloc(&w->dres, sizeof(double) * 3 * n));
     QCD_CUDA_CHECK(cudaMallocHost(&w->h_res, sizeof(double) * 3 * n));
+    QCD_CUDA_CHECK(cudaMalloc(&w->d_field, sizeof(LatField) * 2 * n));
+    QCD_CUDA_CHECK(cudaMallocHost(&w->h_field, sizeof(LatField) * 2 * n));
     QCD_CUDA_CHECK(cudaMalloc(&w->d_status, sizeof(int)));
     QCD_CUDA_CHECK(cudaMemset(w->d_status, 0, sizeof(int)));
     for (int i = 0; i < n; ++i) {
@@ -471,10 +477,31 @@ int ragged_solve(const std::vector<qcd_ctx*>& ctx, RaggedWS*& wp, double* const*
   QCD_CUDA_CHECK(cudaStreamSynchronize(user_st));  // inputs ready
   const dim3 rgrid(w->nblocks, n);
   const Seg seg64{0, w->d_n2off, w->d_n2len};
-  for (int i = 0; i < n; ++i) {
-    int rc = qcd_import_spinor(ctx[i], w->b64 + w->n2off[i], b[i], QCD_PREC_DOUBLE, 1, on_device, (void*)st);
-    if (rc != QCD_OK) throw Error{rc, "lattice " + std::to_string(i) + ": " + ctx[i]->err};
+  // device fields go through one launch over every lattice, host fields
+  // lattice by lattice
+  auto failed = [](int i, int rc, const std::string& what) {
+    throw Error{rc, "lattice " + std::to_string(i) + ": " + what};
+  };
+  auto import_all = [&](const double* const* p, bool to_b) {
+    if (on_device) {
+      LaunchScope ls(c0, QCD_KC_OTHER, st);
+      lat_import_launch(w->d_lat, w->d_site_lat, w->site_blocks, w->d_field + (to_b ? 0 : n), to_b, st);
+      return;
+    }
+    for (int i = 0; i < n; ++i) {
+      int rc = qcd_import_spinor(ctx[i], (to_b ? w->b64 : w->x64) + w->n2off[i], p[i], QCD_PREC_DOUBLE, 1, 0, (void*)st);
+      if (rc != QCD_OK) failed(i, rc, ctx[i]->err);
+    }
+  };
+  if (on_device) {
+    for (int i = 0; i < n; ++i) {
+      const int paper = ctx[i]->basis == QCD_BASIS_PAPER;
+      w->h_field[i] = LatField{const_cast<double*>(b[i]), paper};
+      w->h_field[n + i] = LatField{x[i], paper};
+    }
+    QCD_CUDA_CHECK(cudaMemcpyAsync(w->d_field, w->h_field, sizeof(LatField) * 2 * n, cudaMemcpyHostToDevice, st));
   }
+  import_all(b, true);
   QCD_CUDA_CHECK(cudaMemsetAsync(w->d_status, 0, sizeof(int), st));
   {
     LaunchScope ls(c0, QCD_KC_DOUBLE, st);
@@ -499,10 +526,7 @@ int ragged_solve(const std::vector<qcd_ctx*>& ctx, RaggedWS*& wp, double* const*
     check_launch();
   };
   if (P.x_is_guess) {
-    for (int i = 0; i < n; ++i) {
-      int rc = qcd_import_spinor(ctx[i], w->x64 + w->n2off[i], x[i], QCD_PREC_DOUBLE, 1, on_device, (void*)st);
-      if (rc != QCD_OK) throw Error{rc, "lattice " + std::to_string(i) + ": " + ctx[i]->err};
-    }
+    import_all(x, false);
     residual();
   } else {
     QCD_CUDA_CHECK(cudaMemsetAsync(w->x64, 0, sizeof(double2) * w->n2tot, st));
@@ -570,9 +594,14 @@ int ragged_solve(const std::vector<qcd_ctx*>& ctx, RaggedWS*& wp, double* const*
     QCD_CUDA_CHECK(cudaStreamSynchronize(st));
     for (int i = 0; i < n; ++i) r2[i] = w->h_res[n + i];
   }
-  for (int i = 0; i < n; ++i) {
-    int rc = qcd_export_spinor(ctx[i], x[i], w->x64 + w->n2off[i], QCD_PREC_DOUBLE, 1, on_device, (void*)st);
-    if (rc != QCD_OK) throw Error{rc, "lattice " + std::to_string(i) + ": " + ctx[i]->err};
+  if (on_device) {
+    LaunchScope ls(c0, QCD_KC_OTHER, st);
+    lat_export_launch(w->d_lat, w->d_site_lat, w->site_blocks, w->d_field + n, st);
+  } else {
+    for (int i = 0; i < n; ++i) {
+      int rc = qcd_export_spinor(ctx[i], x[i], w->x64 + w->n2off[i], QCD_PREC_DOUBLE, 1, 0, (void*)st);
+      if (rc != QCD_OK) failed(i, rc, ctx[i]->err);
+    }
   }
   QCD_CUDA_CHECK(cudaStreamSynchronize(st));
   const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
