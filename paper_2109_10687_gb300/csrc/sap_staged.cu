@@ -1,7 +1,6 @@
 // SAP half-sweep kernel for 4^4 domains with the domain's links and C_inv
 // staged in shared memory by bulk asynchronous copies (Sec. 3 of
-// arXiv:2109.10687, Algorithms 1 and 2; the arithmetic is that of
-// sap.cu's generic kernel).
+// arXiv:2109.10687, Algorithms 1 and 2).
 //
 // One CTA per domain, one thread per site, the domain shape fixed at compile
 // time (strides 1, 4, 16, 64).  At entry one thread arms an mbarrier and
