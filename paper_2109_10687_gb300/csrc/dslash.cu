@@ -13,6 +13,7 @@
 
 namespace qcd {
 
+template <bool D4>
 __global__ void __launch_bounds__(192, 4) dslash_df64_split_kernel(Geom g, DF64Spinor out, DF64Spinor in,
                                                                 LinkPtr<df64> U, CloverPtrDF64 clov, df64 kappa,
                                                                 int nrhs);
@@ -240,7 +241,9 @@ void dslash_launch(qcd_ctx* ctx, void* out, const void* in, int prec, int mode, 
     LaunchScope ls(ctx, QCD_KC_DOUBLE, st);
     const long long blocks = (long long)((g.vol + 63) / 64) * nrhs;
     QCD_REQUIRE(blocks < (1LL << 31), QCD_ERR_ARG, "lattice too large for one launch");
-    dslash_df64_split_kernel<<<(unsigned)blocks, dim3(32, 3, 2), 0, st>>>(
+    const bool d4 = g.d[0] == 4 && g.d[1] == 4 && g.d[2] == 4 && g.d[3] == 4;
+    auto kernel = d4 ? dslash_df64_split_kernel<true> : dslash_df64_split_kernel<false>;
+    kernel<<<(unsigned)blocks, dim3(32, 3, 2), 0, st>>>(
         g, DF64Spinor{(float4*)out}, DF64Spinor{(float4*)in}, LinkPtr<df64>{ctx->udf}, CloverPtrDF64{ctx->clovdf},
         df64(ctx->kappa), nrhs);
     check_launch();
@@ -335,20 +338,32 @@ constexpr int DF_SITES = 64;
 // Code size matters more than anything else here: written out for all
 // eight hops and three colour rows, a thread's double-float arithmetic is
 // several thousand instructions that the instruction cache cannot hold, and
-// the warps wait on instruction fetch.  So the hops run in a loop: the
-// neighbour lookup, the loads and the complex multiply-adds are one piece
-// of code for every hop, and only the spin projection and reconstruction,
-// which differ by direction, go through a switch to their fixed forms; the
-// clover rows read their entries by a row index known at run time.  The
-// arithmetic and its order are those of the fully written-out form.
+// the warps wait on instruction fetch.  So the directions run in a loop: the
+// neighbour lookup, the loads and the complex multiply-adds of a direction's
+// two hops are one piece of code for all four, and only the spin projection
+// and reconstruction go through a switch to their fixed forms; the clover
+// rows read their entries by a row index known at run time.  The arithmetic
+// and its order are those of the fully written-out form.
+//
+// Beyond that, issue bounds it, and a third of the instructions were not
+// arithmetic.  32^4: 0.958 ms with a loop over eight hops and strides known
+// at run time; 0.883 with the strides of 4^4 blocks compiled in; 0.829 with a
+// thread's two rows of a chiral block sharing x's loads; 0.784 with the
+// conjugated entries by sign and not by a second body.  The loop over four
+// directions is 0.791 there and 0.456 instead of 0.493 ms in the batch of
+// ragged lattices (0.567 before).
 
 // neighbour (domain, site, sign) of hop (mu, fwd), selected without branches
+// (D4: the strides of 4^4 blocks; mu is known at run time, so they are
+// computed and not looked up in a fixed geometry)
+template <bool D4>
 __device__ __forceinline__ void df_nbr(const Geom& g, int mu, bool fwd, int dom, int s, const int nb[8], int tf,
                                        int& nd, int& ns, bool& neg) {
-  const int c = (s >> g.shift[mu]) & (g.d[mu] - 1);
-  const int step = 1 << g.shift[mu];
-  const int span = (g.d[mu] - 1) * step;
-  const bool inside = fwd ? c < g.d[mu] - 1 : c > 0;
+  const int shift = D4 ? 2 * mu : g.shift[mu], d = D4 ? 4 : g.d[mu];
+  const int c = (s >> shift) & (d - 1);
+  const int step = 1 << shift;
+  const int span = (d - 1) * step;
+  const bool inside = fwd ? c < d - 1 : c > 0;
   const int k = 2 * mu + (fwd ? 0 : 1);
   nd = inside ? dom : nb[k];
   ns = inside ? (fwd ? s + step : s - step) : (fwd ? s - span : s + span);
@@ -365,34 +380,34 @@ __device__ __forceinline__ void df_proj(const cx<df64> q[4], cx<df64>& h0, cx<df
 }
 
 // phase 1 loads: colour a of the four spins of hop's neighbour, and its sign
+template <bool D4>
 __device__ __forceinline__ void df_project_load(const Geom& g, const DF64Spinor& in, int hop, int dom, int s, int a,
                                                 const int nb[8], int tf, float4 q[4], bool& neg) {
   int nd, ns;
-  df_nbr(g, hop >> 1, !(hop & 1), dom, s, nb, tf, nd, ns, neg);
+  df_nbr<D4>(g, hop >> 1, !(hop & 1), dom, s, nb, tf, nd, ns, neg);
+  const int logvd = D4 ? 8 : g.logvd;
 #pragma unroll
-  for (int sp = 0; sp < 4; ++sp) q[sp] = __ldg(in.p + in.idx(g, nd, sp * 3 + a, ns));
+  for (int sp = 0; sp < 4; ++sp) q[sp] = __ldg(in.p + ((size_t)(nd * 12 + sp * 3 + a) << logvd) + ns);
 }
 
 // phase 1: rows (h0, h1) of colour a of the projected neighbour, signed
-__device__ __forceinline__ void df_project(int hop, int a, const float4 qv[4], bool neg, float4* sh, int sl) {
+template <bool FWD>
+__device__ __forceinline__ void df_project(int mu, int a, const float4 qv[4], bool neg, float4* sh, int sl) {
   cx<df64> q[4];
 #pragma unroll
   for (int sp = 0; sp < 4; ++sp) q[sp] = df_unpack(qv[sp]);
   cx<df64> h0, h1;
-  switch (hop) {
-    case 0: df_proj<0, true>(q, h0, h1); break;
-    case 1: df_proj<0, false>(q, h0, h1); break;
-    case 2: df_proj<1, true>(q, h0, h1); break;
-    case 3: df_proj<1, false>(q, h0, h1); break;
-    case 4: df_proj<2, true>(q, h0, h1); break;
-    case 5: df_proj<2, false>(q, h0, h1); break;
-    case 6: df_proj<3, true>(q, h0, h1); break;
-    default: df_proj<3, false>(q, h0, h1); break;
+  switch (mu) {
+    case 0: df_proj<0, FWD>(q, h0, h1); break;
+    case 1: df_proj<1, FWD>(q, h0, h1); break;
+    case 2: df_proj<2, FWD>(q, h0, h1); break;
+    default: df_proj<3, FWD>(q, h0, h1); break;
   }
   if (neg) {  // exact: a sign flip of both parts
     h0 = make_cx(-h0.re, -h0.im);
     h1 = make_cx(-h1.re, -h1.im);
   }
+  const int hop = 2 * mu + (FWD ? 0 : 1);
   sh[((hop * 2 + 0) * 3 + a) * DF_SITES + sl] = df_pack(h0);
   sh[((hop * 2 + 1) * 3 + a) * DF_SITES + sl] = df_pack(h1);
 }
@@ -420,30 +435,28 @@ __device__ __forceinline__ void df_rebuild(cx<df64> h0, cx<df64> h1, cx<df64> ac
 }
 
 // phase 2 loads: row a (forward) or column a (backward) of hop's link
-__device__ __forceinline__ void df_link_load(const Geom& g, const LinkPtr<df64>& U, int hop, int dom, int s, int a,
+template <bool D4, bool FWD>
+__device__ __forceinline__ void df_link_load(const Geom& g, const LinkPtr<df64>& U, int mu, int dom, int s, int a,
                                              const int nb[8], int tf, float4 v[3]) {
-  const int mu = hop >> 1;
-  const bool fwd = !(hop & 1);
-  int nd, ns;
+  const int logvd = D4 ? 8 : g.logvd;
+  int nd = dom, ns = s;
   bool neg;
-  df_nbr(g, mu, fwd, dom, s, nb, tf, nd, ns, neg);
-  const size_t base = ((size_t)(((fwd ? dom : nd) * 4 + mu) * 9)) << g.logvd;
-  const int site = fwd ? s : ns;
+  if (!FWD) df_nbr<D4>(g, mu, false, dom, s, nb, tf, nd, ns, neg);
+  const float4* p = U.p + (((size_t)((nd * 4 + mu) * 9)) << logvd) + ns;
 #pragma unroll
-  for (int b = 0; b < 3; ++b) {
-    const int e = fwd ? a * 3 + b : b * 3 + a;
-    v[b] = __ldg(U.p + base + ((size_t)e << g.logvd) + site);
-  }
+  for (int b = 0; b < 3; ++b) v[b] = __ldg(p + ((size_t)(FWD ? a * 3 + b : b * 3 + a) << logvd));
 }
 
 // phase 2: row a of U h (forward) or U^dag h (backward), rebuilt into colour a
-__device__ __forceinline__ void df_mul_acc(int hop, const float4 v[3], const float4* sh, int sl, cx<df64> acc[4]) {
-  const bool fwd = !(hop & 1);
+template <bool FWD>
+__device__ __forceinline__ void df_mul_acc(int mu, const float4 v[3], const float4* sh, int sl, cx<df64> acc[4]) {
   cx<df64> row[3];
 #pragma unroll
-  for (int b = 0; b < 3; ++b)
-    row[b] = fwd ? make_cx(df64(v[b].x, v[b].y), df64(v[b].z, v[b].w))
-                 : make_cx(df64(v[b].x, v[b].y), -df64(v[b].z, v[b].w));
+  for (int b = 0; b < 3; ++b) {
+    row[b] = df_unpack(v[b]);
+    if (!FWD) row[b].im = -row[b].im;
+  }
+  const int hop = 2 * mu + (FWD ? 0 : 1);
   cx<df64> uh[2];
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
@@ -452,19 +465,15 @@ __device__ __forceinline__ void df_mul_acc(int hop, const float4 v[3], const flo
     t = cmac(t, row[2], df_unpack(sh[((hop * 2 + r) * 3 + 2) * DF_SITES + sl]));
     uh[r] = t;
   }
-  switch (hop) {
-    case 0: df_rebuild<0, true>(uh[0], uh[1], acc); break;
-    case 1: df_rebuild<0, false>(uh[0], uh[1], acc); break;
-    case 2: df_rebuild<1, true>(uh[0], uh[1], acc); break;
-    case 3: df_rebuild<1, false>(uh[0], uh[1], acc); break;
-    case 4: df_rebuild<2, true>(uh[0], uh[1], acc); break;
-    case 5: df_rebuild<2, false>(uh[0], uh[1], acc); break;
-    case 6: df_rebuild<3, true>(uh[0], uh[1], acc); break;
-    default: df_rebuild<3, false>(uh[0], uh[1], acc); break;
+  switch (mu) {
+    case 0: df_rebuild<0, FWD>(uh[0], uh[1], acc); break;
+    case 1: df_rebuild<1, FWD>(uh[0], uh[1], acc); break;
+    case 2: df_rebuild<2, FWD>(uh[0], uh[1], acc); break;
+    default: df_rebuild<3, FWD>(uh[0], uh[1], acc); break;
   }
 }
 
-// (1 + C) x, row i of block b (i = 3 r + a, known at run time): the block's
+// (1 + C) x, rows 3 r + a (r = 0, 1; a known at run time) of block b: its
 // packed reals come straight from memory, the diagonal one as a real
 // factor and the off-diagonal ones conjugated below the diagonal; the loads
 // of column j + 1 are issued before the arithmetic of column j
@@ -472,35 +481,46 @@ __device__ __forceinline__ float4 df_clover_entry(const float4* cp, int logvd, i
   const int k = j == i ? (i >> 1) : 3 + (j > i ? herm_off(i, j) : herm_off(j, i));
   return __ldg(cp + ((size_t)k << logvd));
 }
-__device__ __forceinline__ cx<df64> df_clover_row(const Geom& g, const DF64Spinor& in, const CloverPtrDF64& clov,
-                                                  int dom, int s, int b, int i) {
-  const float4* cp = clov.p + (((size_t)(dom * 36 + 18 * b)) << g.logvd) + s;
-  cx<df64> y = make_cx(df64(0.f), df64(0.f));
-  float4 xn = __ldg(in.p + in.idx(g, dom, (2 * b) * 3, s));
-  float4 cn = df_clover_entry(cp, g.logvd, i, 0);
+template <bool D4>
+__device__ __forceinline__ void df_clover_rows(const Geom& g, const DF64Spinor& in, const CloverPtrDF64& clov, int dom,
+                                               int s, int b, int a, cx<df64> y[2]) {
+  const int logvd = D4 ? 8 : g.logvd;
+  const float4* cp = clov.p + (((size_t)(dom * 36 + 18 * b)) << logvd) + s;
+  const float4* xp = in.p + ((size_t)(dom * 12 + 6 * b) << logvd) + s;
+  float4 xn = __ldg(xp), cn[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    y[r] = make_cx(df64(0.f), df64(0.f));
+    cn[r] = df_clover_entry(cp, logvd, 3 * r + a, 0);
+  }
 #pragma unroll 1
   for (int j = 0; j < 6; ++j) {
-    const float4 xv = xn, cv = cn;
+    const float4 xv = xn, cv[2] = {cn[0], cn[1]};
     if (j < 5) {
-      xn = __ldg(in.p + in.idx(g, dom, (2 * b + (j + 1) / 3) * 3 + (j + 1) % 3, s));
-      cn = df_clover_entry(cp, g.logvd, i, j + 1);
+      xn = __ldg(xp + ((size_t)(j + 1) << logvd));
+#pragma unroll
+      for (int r = 0; r < 2; ++r) cn[r] = df_clover_entry(cp, logvd, 3 * r + a, j + 1);
     }
     const cx<df64> xj = df_unpack(xv);
-    if (j == i) {
-      const df64 d = (i & 1) ? df64(cv.z, cv.w) : df64(cv.x, cv.y);
-      y = make_cx(fma(d, xj.re, y.re), fma(d, xj.im, y.im));
-    } else {
-      const cx<df64> c = df_unpack(cv);
-      y = j > i ? cmac(y, c, xj) : cmacc(y, c, xj);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int i = 3 * r + a;
+      if (j == i) {
+        const df64 d = (i & 1) ? df64(cv[r].z, cv[r].w) : df64(cv[r].x, cv[r].y);
+        y[r] = make_cx(fma(d, xj.re, y[r].re), fma(d, xj.im, y[r].im));
+      } else {
+        cx<df64> c = df_unpack(cv[r]);
+        if (j < i) c.im = -c.im;  // conjugated below the diagonal
+        y[r] = cmac(y[r], c, xj);
+      }
     }
   }
-  return y;
 }
 
 // One tile of DF_SITES sites from site0 (lexicographic-domain order) of the
 // field `in` (one right-hand side); every thread of the block takes part.
 // store(dom, comp, s, value) writes one colour row of the result.
-template <typename Store>
+template <bool D4, typename Store>
 __device__ __forceinline__ void df64_tile(const Geom& g, const DF64Spinor& inr, const LinkPtr<df64>& U,
                                           const CloverPtrDF64& clov, df64 kappa, long long site0, float4* sh,
                                           const Store& store) {
@@ -511,8 +531,8 @@ __device__ __forceinline__ void df64_tile(const Geom& g, const DF64Spinor& inr, 
   // site 0 of the block's range and store nothing
   const bool live = gid < g.vol;
   const long long gq = live ? gid : site0;
-  const int dom = __ldg(g.lex2dom + (int)(gq >> g.logvd));
-  const int s = (int)(gq & (g.vd - 1));
+  const int dom = __ldg(g.lex2dom + (int)(gq >> (D4 ? 8 : g.logvd)));
+  const int s = (int)(gq & ((D4 ? 256 : g.vd) - 1));
   int nb[8];
   {
     const int4 n0 = __ldg(reinterpret_cast<const int4*>(g.nbr) + 2 * dom);
@@ -523,17 +543,15 @@ __device__ __forceinline__ void df64_tile(const Geom& g, const DF64Spinor& inr, 
   const int tf = __ldg(g.tflag + dom);
   // each loop issues the next hop's loads before this hop's arithmetic
   {
-    float4 qn[4];
-    bool negn;
-    df_project_load(g, inr, 0, dom, s, a, nb, tf, qn, negn);
+    float4 qf[4], qb[4];
+    bool nf, nbk;
+    df_project_load<D4>(g, inr, 0, dom, s, a, nb, tf, qf, nf);
 #pragma unroll 1
-    for (int hop = 0; hop < 8; ++hop) {
-      float4 q[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) q[k] = qn[k];
-      const bool neg = negn;
-      if (hop < 7) df_project_load(g, inr, hop + 1, dom, s, a, nb, tf, qn, negn);
-      df_project(hop, a, q, neg, sh, sl);
+    for (int mu = 0; mu < 4; ++mu) {
+      df_project_load<D4>(g, inr, 2 * mu + 1, dom, s, a, nb, tf, qb, nbk);
+      df_project<true>(mu, a, qf, nf, sh, sl);
+      if (mu < 3) df_project_load<D4>(g, inr, 2 * mu + 2, dom, s, a, nb, tf, qf, nf);
+      df_project<false>(mu, a, qb, nbk, sh, sl);
     }
   }
   __syncthreads();
@@ -541,29 +559,27 @@ __device__ __forceinline__ void df64_tile(const Geom& g, const DF64Spinor& inr, 
 #pragma unroll
   for (int sp = 0; sp < 4; ++sp) acc[sp] = make_cx(df64(0.f), df64(0.f));
   {
-    float4 vn[3];
-    df_link_load(g, U, 0, dom, s, a, nb, tf, vn);
+    float4 vf[3], vb[3];
+    df_link_load<D4, true>(g, U, 0, dom, s, a, nb, tf, vf);
 #pragma unroll 1
-    for (int hop = 0; hop < 8; ++hop) {
-      float4 v[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) v[k] = vn[k];
-      if (hop < 7) df_link_load(g, U, hop + 1, dom, s, a, nb, tf, vn);
-      df_mul_acc(hop, v, sh, sl, acc);
+    for (int mu = 0; mu < 4; ++mu) {
+      df_link_load<D4, false>(g, U, mu, dom, s, a, nb, tf, vb);
+      df_mul_acc<true>(mu, vf, sh, sl, acc);
+      if (mu < 3) df_link_load<D4, true>(g, U, mu + 1, dom, s, a, nb, tf, vf);
+      df_mul_acc<false>(mu, vb, sh, sl, acc);
     }
   }
   if (!live) return;
   // (1 + C) x, rows (block b, spin-in-block r, colour a): index i = 3 r + a
   cx<df64> res[4];
 #pragma unroll
-  for (int b = 0; b < 2; ++b)
-#pragma unroll
-    for (int r = 0; r < 2; ++r) res[2 * b + r] = df_clover_row(g, inr, clov, dom, s, b, 3 * r + a);
+  for (int b = 0; b < 2; ++b) df_clover_rows<D4>(g, inr, clov, dom, s, b, a, res + 2 * b);
 #pragma unroll
   for (int sp = 0; sp < 4; ++sp)
     store(dom, sp * 3 + a, s, make_cx(fma(-kappa, acc[sp].re, res[sp].re), fma(-kappa, acc[sp].im, res[sp].im)));
 }
 
+template <bool D4>
 __global__ void __launch_bounds__(192, 4) dslash_df64_split_kernel(Geom g, DF64Spinor out, DF64Spinor in,
                                                                 LinkPtr<df64> U, CloverPtrDF64 clov, df64 kappa,
                                                                 int nrhs) {
@@ -571,7 +587,7 @@ __global__ void __launch_bounds__(192, 4) dslash_df64_split_kernel(Geom g, DF64S
   const int rhs = blockIdx.x % nrhs;
   const int rhs_off = rhs * g.ndom;
   const DF64Spinor inr{in.p + ((size_t)rhs_off * 12 << g.logvd)};
-  df64_tile(g, inr, U, clov, kappa, (blockIdx.x / nrhs) * (long long)DF_SITES, sh,
+  df64_tile<D4>(g, inr, U, clov, kappa, (blockIdx.x / nrhs) * (long long)DF_SITES, sh,
             [&](int dom, int comp, int s, cx<df64> o) { out.p[out.idx(g, dom + rhs_off, comp, s)] = df_pack(o); });
 }
 
@@ -596,7 +612,8 @@ __global__ void __launch_bounds__(192, 4) lat_dslash_df64_kernel(const LatDesc* 
   const int kexp = df_scale_exp(b2[lat], (size_t)sd.g.vol * 12);
   const F64Spinor out{sd.r64};
   const Geom& g = sd.g;
-  df64_tile(g, DF64Spinor{sd.xdf}, LinkPtr<df64>{sd.udf}, CloverPtrDF64{sd.clovdf}, df64(sd.kappa64),
+  // every lattice of the shared solve has 4^4 domains
+  df64_tile<true>(g, DF64Spinor{sd.xdf}, LinkPtr<df64>{sd.udf}, CloverPtrDF64{sd.clovdf}, df64(sd.kappa64),
             ((long long)blockIdx.x - sd.df_tile_begin) * DF_SITES, dsh, [&](int dom, int comp, int s, cx<df64> o) {
               out.p[out.idx(g, dom, comp, s)] =
                   make_double2(df64_to_double_scaled(o.re, kexp), df64_to_double_scaled(o.im, kexp));
