@@ -661,6 +661,21 @@ __device__ __forceinline__ void clover_mul(const Ptr& cp, const Geom& g, int dom
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Start of a kernel of an M_SAP sequence: true if it has nothing to do (the
+// loop's flag, or the lattice's own `skip`), else the next launch may start.
+// The flags are the BLAS kernels' before the sequence, and before the wait
+// their last writes need not be visible: every thread of the grid would not
+// take the same decision, and those that go on would wait for those that left.
+// So the sequence's first launch (`first`) waits before it reads them and
+// before it lets the next one start, which then finds them settled; no launch
+// of the sequence writes them.
+__device__ __forceinline__ bool pdl_enter(const Geom& g, bool first, const int* skip = nullptr) {
+  if (first && (g.run_flag || skip)) pdl_wait();
+  if (loop_idle(g) || (skip && *(volatile const int*)skip)) return true;
+  pdl_trigger();
+  return false;
+}
+
 // ---------------------------------------------------------------------------
 // context (host side)
 // ---------------------------------------------------------------------------

@@ -241,8 +241,7 @@ __global__ void __launch_bounds__(NT, HALF ? 512 / NT : (NT == 64 ? 5 : 256 / NT
   Link* sl = reinterpret_cast<Link*>(sx + 6 * (NT + SB_GHOST));
   unsigned char* sc = reinterpret_cast<unsigned char*>(sl) + (size_t)NT * BlockOp<HALF>::LINK_BYTES;
   const Geom& g = a.g;
-  if (loop_idle(g)) return;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (pdl_enter(g, !a.do_surface)) return;
   const int l = threadIdx.x;
   const int total = g.nhalf << g.logvd, first = blockIdx.x * NT;
   const int nsites = min(NT, total - first);  // whole domains

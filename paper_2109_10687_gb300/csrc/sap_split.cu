@@ -234,9 +234,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
   __shared__ float4 zero4;
   __shared__ float nrm[4 * SP_SITES];
   const Geom& g = a.g;
-  // the same decision in every block: the flag was written before this launch
-  if (loop_idle(g)) return;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (pdl_enter(g, !a.do_surface)) return;  // the same decision in every block of the cluster
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // direction in the hops, spin in the site sums
   const int q = w >> 1, site = (w & 1) * 32 + lane;

@@ -693,10 +693,9 @@ __device__ __forceinline__ bool sap_staged_item(const StagedArgs<HALF, SIO>& a, 
 // one launch = one half-sweep: the launch's mode and the CTA's domain
 template <bool HALF, typename SIO, int SPT>
 __device__ __forceinline__ void sap_staged_body(const StagedArgs<HALF, SIO>& a, int blk) {
-  if (loop_idle(a.g) || (a.skip && *(volatile const int*)a.skip)) return;
   // programmatic dependent launch: the next launch in the stream may start
   // its CTAs while this grid drains
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (pdl_enter(a.g, !a.do_surface, a.skip)) return;
   int hcount = 0;
   sap_staged_item<HALF, SIO, SPT>(a, launch_mode(a), blk, 0, hcount, true, true, false);
 }
@@ -768,8 +767,7 @@ __global__ void __launch_bounds__(ST_THREADS, HALF ? 2 : 1) sap_flow_kernel(Stag
   uint64_t* lbar = reinterpret_cast<uint64_t*>(sc + ST::CLOV_BYTES);
   __shared__ int s_item, s_next, s_last;
   const Geom& g = a.g;
-  if (loop_idle(g) || (a.skip && *(volatile const int*)a.skip)) return;  // the same for every CTA
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (pdl_enter(g, true, a.skip)) return;  // the same for every CTA
   // The counters and flags belong to the previous use until its grid has
   // completed, and the earlier launches' outputs are read below: wait for
   // the previous grid (which itself waited for its own predecessor) first.

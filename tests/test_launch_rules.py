@@ -1,0 +1,50 @@
+"""Rules of the kernels' launches that no run on one idle GPU can show broken,
+checked in the sources."""
+
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2109_10687_gb300", "csrc")
+FILES = sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")))
+
+
+def _code(path):
+    text = open(path).read()
+    return re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+
+
+def _functions(code):
+    """(head, body) of every device function and kernel."""
+    for m in re.finditer(r"__(?:global|device)__[^;{]*\{", code):
+        depth, i = 1, m.end()
+        while depth and i < len(code):
+            depth += {"{": 1, "}": -1}.get(code[i], 0)
+            i += 1
+        yield m.group(0), code[m.end():i]
+
+
+WAIT = re.compile(r"pdl_wait\(\)|griddepcontrol\.wait")
+TRIGGER = re.compile(r"pdl_trigger\(\)|griddepcontrol\.launch_dependents")
+FLAG = re.compile(r"loop_idle\(|\bskip\s*&&")
+
+
+@pytest.mark.parametrize("path", FILES, ids=os.path.basename)
+def test_flags_of_the_loop_are_read_where_they_are_visible(path):
+    """A kernel that may start before its predecessor has finished reads the
+    loop's flags after its wait, or through pdl_enter, which waits in a
+    sequence's first launch.  The cluster kernel's first launch is a plain one."""
+    for head, body in _functions(_code(path)):
+        if "pdl_enter" in head or "sap_cluster_kernel" in head:
+            continue
+        if not (WAIT.search(body) or TRIGGER.search(body)):
+            continue  # never launched early
+        for m in FLAG.finditer(body):
+            assert WAIT.search(body, 0, m.start()), head
+
+
+def test_the_first_launch_of_the_cluster_kernel_is_a_plain_one():
+    code = _code(os.path.join(CSRC, "sap_cluster.cu"))
+    assert re.search(r"numAttrs = with_halo && \(r > 0 \|\| sweep > 0 \|\| colour > 0\) \? 2 : 1;", code)
