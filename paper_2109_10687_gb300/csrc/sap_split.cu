@@ -195,23 +195,6 @@ __device__ __forceinline__ void sp_gather(const float2* hs, int site, cx<float> 
     sp_take<3, +1, Q, false>(hs, site, acc);
   }
 }
-// y = spin Q of C_inv (the sum of the hops); two barriers
-template <bool SURFACE, int Q>
-__device__ __forceinline__ void sp_site_sum(const float2* hs, float2* ex, const CinvRows& m, int site,
-                                            cx<float> y[3]) {
-  cx<float> acc[3], oth[3];
-  sp_gather<SURFACE, Q>(hs, site, acc);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) ex[(Q * 3 + c) * SP_SITES + site] = make_float2(acc[c].re, acc[c].im);
-  __syncthreads();
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const float2 v = ex[((Q ^ 1) * 3 + c) * SP_SITES + site];
-    oth[c] = make_cx(v.x, v.y);
-  }
-  sp_cinv_mul<(Q & 1)>(m, acc, oth, y);
-}
-
 // f(k) for the warp-uniform k = 0..3 as a compile-time constant
 template <typename F>
 __device__ __forceinline__ void sp_switch(int k, F f) {
@@ -219,6 +202,25 @@ __device__ __forceinline__ void sp_switch(int k, F f) {
   else if (k == 1) f(std::integral_constant<int, 1>{});
   else if (k == 2) f(std::integral_constant<int, 2>{});
   else f(std::integral_constant<int, 3>{});
+}
+
+// y = spin q of C_inv (the sum of the hops).  One barrier, outside the
+// switches: q differs between the warps of a block.
+template <bool SURFACE>
+__device__ __forceinline__ void sp_site_sum(const float2* hs, float2* ex, const CinvRows& m, int q, int site,
+                                            cx<float> y[3]) {
+  cx<float> acc[3], oth[3];
+  sp_switch(q, [&](auto k) { sp_gather<SURFACE, decltype(k)::value>(hs, site, acc); });
+#pragma unroll
+  for (int c = 0; c < 3; ++c) ex[(q * 3 + c) * SP_SITES + site] = make_float2(acc[c].re, acc[c].im);
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float2 v = ex[((q ^ 1) * 3 + c) * SP_SITES + site];
+    oth[c] = make_cx(v.x, v.y);
+  }
+  if (q & 1) sp_cinv_mul<1>(m, acc, oth, y);
+  else sp_cinv_mul<0>(m, acc, oth, y);
 }
 
 // component comp = spin * 3 + colour of a float32 field
@@ -300,7 +302,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
       sp_hop_bwd<MU>(ub, p, bsign, hs, site);
     });
     __syncthreads();
-    sp_switch(q, [&](auto k) { sp_site_sum<true, decltype(k)::value>(hs, ex, m, site, y); });
+    sp_site_sum<true>(hs, ex, m, q, site, y);
 #pragma unroll
     for (int c = 0; c < 3; ++c) src[c] = cfma(a.kappa, y[c], src[c]);
   }
@@ -321,7 +323,7 @@ __global__ void __launch_bounds__(SP_THREADS, 2) sap_split_kernel(SplitArgs<HALF
       sp_hop_bwd<MU>(ub, p, 1.f, hs, site);
     });
     __syncthreads();
-    sp_switch(q, [&](auto k) { sp_site_sum<false, decltype(k)::value>(hs, ex, m, site, y); });
+    sp_site_sum<false>(hs, ex, m, q, site, y);
     if (it < a.n_jac) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) xk[c] = cfma(a.kappa, y[c], src[c]);

@@ -48,3 +48,27 @@ def test_flags_of_the_loop_are_read_where_they_are_visible(path):
 def test_the_first_launch_of_the_cluster_kernel_is_a_plain_one():
     code = _code(os.path.join(CSRC, "sap_cluster.cu"))
     assert re.search(r"numAttrs = with_halo && \(r > 0 \|\| sweep > 0 \|\| colour > 0\) \? 2 : 1;", code)
+
+
+@pytest.mark.parametrize("path", FILES, ids=os.path.basename)
+def test_no_block_barrier_under_a_choice_per_warp(path):
+    """What runs under sp_switch differs between the warps of a block: no
+    function called there, nor the lambda itself, holds a block barrier."""
+    code = _code(path)
+    bodies = {}
+    for head, body in _functions(code):
+        name = re.findall(r"(\w+)\s*\(", head)
+        if name:
+            bodies.setdefault(name[-1] if "__launch_bounds__" in head else name[0], []).append(body)
+    for m in re.finditer(r"sp_switch\(\w+, \[&\]\(auto k\) \{", code):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(code[i], 0)
+            i += 1
+        todo, seen = [code[m.end():i]], set()
+        while todo:
+            body = todo.pop()
+            assert "__syncthreads" not in body and "cl.sync" not in body, body
+            for callee in set(re.findall(r"\b(\w+)(?:<[^;{}]*?>)?\(", body)) & set(bodies) - seen:
+                seen.add(callee)
+                todo += bodies[callee]
