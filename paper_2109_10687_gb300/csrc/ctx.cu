@@ -453,6 +453,7 @@ extern "C" int qcd_create(const int dims[4], const int domain[4], int bc_t, int 
     g.bc_t = bc_t;
     ctx->basis = basis;
     QCD_CUDA_CHECK(cudaGetDevice(&ctx->device));
+    QCD_CUDA_CHECK(cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device));
 
     // domain neighbour table, colour-major domain numbering
     std::vector<int> id_of_lex(g.ndom), nbr((size_t)g.ndom * 8);

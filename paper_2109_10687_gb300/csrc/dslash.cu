@@ -624,11 +624,8 @@ void lat_dslash_df64_launch(const LatDesc* d_lat, const int* d_tile_lat, long lo
                             cudaStream_t st) {
   QCD_REQUIRE(tiles < (1LL << 31), QCD_ERR_ARG, "batch too large for one launch");
   const int smem = (int)(sizeof(float4) * 8 * 2 * 3 * DF_SITES + sizeof(LatDesc));
-  static const bool attr = [smem] {
-    QCD_CUDA_CHECK(cudaFuncSetAttribute(lat_dslash_df64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    return true;
-  }();
-  (void)attr;
+  // the limit is the current device's
+  QCD_CUDA_CHECK(cudaFuncSetAttribute(lat_dslash_df64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   lat_dslash_df64_kernel<<<(unsigned)tiles, dim3(32, 3, 2), smem, st>>>(d_lat, d_tile_lat, d_b2);
   check_launch();
 }

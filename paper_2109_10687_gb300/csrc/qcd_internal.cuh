@@ -689,6 +689,7 @@ struct qcd_ctx {
   qcd::Geom geom;
   int basis = QCD_BASIS_CHIRAL;
   int device = 0;
+  int sms = 0;                   // SMs of the device
   double kappa = 0.125, csw = 1.0;
   bool have_gauge = false, have_clover = false;
   // device arrays owned by the context

@@ -339,27 +339,17 @@ __global__ void __launch_bounds__(NT, HALF ? 512 / NT : (NT == 64 ? 5 : 256 / NT
   if (live) a.x.store(g, domr, s, xk);
 }
 
-template <bool HALF, typename SIO, int NT>
-static void block_launch(const BlockArgs<HALF, SIO>& a, int nrhs, cudaStream_t st) {
-  static const bool attr = [] {
-    QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_block_kernel<HALF, SIO, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)sb_smem<HALF, NT>()));
-    return true;
-  }();
-  (void)attr;
-  const long long sites = (long long)a.g.nhalf << a.g.logvd;
-  QCD_REQUIRE(sites + NT < (1LL << 31), QCD_ERR_ARG, "SAP: lattice too large");
-  launch_pdl(sap_block_kernel<HALF, SIO, NT>, dim3((unsigned)((sites + NT - 1) / NT), nrhs), dim3(NT),
-             sb_smem<HALF, NT>(), st, a);
-  check_launch();
-}
-
 // Algorithm 1 as 2 (n_sap + 1) launches, every right-hand side in each.
 // b: the source, also the first sweep's input; x: the result, which holds the
 // iterates of both colours on the way.
-template <bool HALF, typename SIO>
-static void block_sequence(qcd_ctx* ctx, SIO s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
+template <bool HALF, typename SIO, int NT>
+static void block_launches(qcd_ctx* ctx, SIO s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
                            cudaStream_t st) {
+  const long long sites = (long long)ctx->geom.nhalf << ctx->geom.logvd;
+  QCD_REQUIRE(sites + NT < (1LL << 31), QCD_ERR_ARG, "SAP: lattice too large");
+  // the limit is the current device's, and a process may use several
+  QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_block_kernel<HALF, SIO, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sb_smem<HALF, NT>()));
   BlockArgs<HALF, SIO> a;
   a.g = ctx->geom;
   a.n_jac = n_jac;
@@ -377,11 +367,19 @@ static void block_sequence(qcd_ctx* ctx, SIO s, F32Spinor x, F32Spinor b, int nr
       a.colour = colour;
       a.do_surface = (sweep == 0 && colour == 0) ? 0 : 1;
       LaunchScope ls(ctx, QCD_KC_SAP_BLOCK, st);
-      if (a.g.vd <= 64) block_launch<HALF, SIO, 64>(a, nrhs, st);
-      else if (a.g.vd == 128) block_launch<HALF, SIO, 128>(a, nrhs, st);
-      else block_launch<HALF, SIO, 256>(a, nrhs, st);
+      launch_pdl(sap_block_kernel<HALF, SIO, NT>, dim3((unsigned)((sites + NT - 1) / NT), nrhs), dim3(NT),
+                 sb_smem<HALF, NT>(), st, a);
+      check_launch();
     }
   }
+}
+template <bool HALF, typename SIO>
+static void block_sequence(qcd_ctx* ctx, SIO s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,
+                           cudaStream_t st) {
+  const int vd = ctx->geom.vd;
+  if (vd <= 64) block_launches<HALF, SIO, 64>(ctx, s, x, b, nrhs, n_sap, n_jac, st);
+  else if (vd == 128) block_launches<HALF, SIO, 128>(ctx, s, x, b, nrhs, n_sap, n_jac, st);
+  else block_launches<HALF, SIO, 256>(ctx, s, x, b, nrhs, n_sap, n_jac, st);
 }
 
 void sap_block_f32(qcd_ctx* ctx, F32Spinor s, F32Spinor x, F32Spinor b, int nrhs, int n_sap, int n_jac,

@@ -930,14 +930,8 @@ constexpr int st_smem_bytes() {
 // blocks a launch: 0.229 -> 0.142 ms).
 constexpr int ST_ONE_PER_SM = 120 * 1024;
 template <bool HALF>
-static int st_launch_smem(long long blocks) {
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    QCD_CUDA_CHECK(cudaGetDevice(&dev));
-    QCD_CUDA_CHECK(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-    return n;
-  }();
-  return HALF && blocks <= sms ? ST_ONE_PER_SM : st_smem_bytes<HALF>();
+static int st_launch_smem(const qcd_ctx* ctx, long long blocks) {
+  return HALF && blocks <= ctx->sms ? ST_ONE_PER_SM : st_smem_bytes<HALF>();
 }
 
 void sap_staging_alloc(qcd_ctx* ctx) {
@@ -1022,7 +1016,7 @@ static void staged_sequence_shape(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, S
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(ctx->geom.nhalf, rhs_grid ? nrhs : 1);
       cfg.blockDim = dim3(ST_THREADS / SPT);
-      cfg.dynamicSmemBytes = st_launch_smem<HALF>((long long)cfg.gridDim.x * cfg.gridDim.y);
+      cfg.dynamicSmemBytes = st_launch_smem<HALF>(ctx, (long long)cfg.gridDim.x * cfg.gridDim.y);
       cfg.stream = st;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1067,18 +1061,17 @@ static void flow_sequence(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, SIO x, F3
   f.ctr = ctx->flow_state;
   f.n_sap = n_sap;
   f.stagger_ns = stagger_ns;
-  // as many CTAs as can be resident at once (computed once; the batch
-  // solve's host threads may get here together)
-  static const int resident = [] {
-    int dev = 0, sms = 0, per_sm = 0;
-    QCD_CUDA_CHECK(cudaGetDevice(&dev));
-    QCD_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    QCD_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sap_flow_kernel<HALF, SIO>, ST_THREADS,
+  // as many CTAs as can be resident at once (those of an SM, the same on every
+  // device the library runs on, computed once; the batch solve's host threads
+  // may get here together)
+  static const int per_sm = [] {
+    int n = 0;
+    QCD_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sap_flow_kernel<HALF, SIO>, ST_THREADS,
                                                                  st_smem_bytes<HALF>()));
-    return per_sm * sms;
+    return n;
   }();
   const int total = 2 * (n_sap + 1) * ctx->geom.nhalf;
-  const int grid = std::max(1, std::min(total, resident));
+  const int grid = std::max(1, std::min(total, per_sm * ctx->sms));
   LaunchScope ls(ctx, QCD_KC_SAP_BLOCK, st);
   launch_pdl(sap_flow_kernel<HALF, SIO>, dim3(grid), dim3(ST_THREADS), st_smem_bytes<HALF>(), st, a, f);
   check_launch();

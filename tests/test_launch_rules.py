@@ -72,3 +72,11 @@ def test_no_block_barrier_under_a_choice_per_warp(path):
             for callee in set(re.findall(r"\b(\w+)(?:<[^;{}]*?>)?\(", body)) & set(bodies) - seen:
                 seen.add(callee)
                 todo += bodies[callee]
+
+
+@pytest.mark.parametrize("path", FILES, ids=os.path.basename)
+def test_device_settings_are_not_kept_per_process(path):
+    """A kernel's shared-memory limit and a device's properties belong to the
+    current device: no function-local static sets or holds them."""
+    for m in re.finditer(r"static (?:const )?\w+ \w+ = \[[^\]]*\][^{]*\{(.*?)\}\(\);", _code(path), flags=re.S):
+        assert not re.search(r"cudaFuncSetAttribute|cudaDeviceGetAttribute|cudaGetDevice", m.group(1)), m.group(0)
