@@ -150,8 +150,8 @@ const char* qcd_version(void);
  * context in float64, float32 and float16 internal layouts.  U_mu(n) is the
  * SU(3) link from n to n + mu (App. A; U_{-mu}(n) = U_mu(n - mu)^dag).
  * on_device: 1 if U is a device pointer, 0 for host memory.
- * check_tol > 0: reject links with |U^dag U - 1| or |det U - 1| above it
- * (QCD_ERR_ARG).  Invalidates a previously built clover term. */
+ * check_tol > 0: reject links with |U^dag U - 1| or |det U - 1| above it or
+ * with entries that are not finite (QCD_ERR_ARG).  Invalidates a previously built clover term. */
 int qcd_set_gauge(qcd_ctx* ctx, const double* U, int on_device, double check_tol, void* stream);
 
 /* Set the hopping parameter kappa and the clover coefficient c_SW (App. A).

@@ -563,6 +563,11 @@ extern "C" int qcd_set_gauge(qcd_ctx* ctx, const double* U, int on_device, doubl
   ctx->have_gauge = true;
   ctx->have_clover = false;
   ctx->su3_links = worst <= 1e-9 && hbad[1] == 0;
+  // NaN entries drop out of the worst deviation (fmax), so they have a word of their own
+  if (check_tol > 0 && hbad[1]) {
+    ctx->have_gauge = false;
+    throw qcd::Error{QCD_ERR_ARG, "qcd_set_gauge: non-finite links"};
+  }
   if (check_tol > 0 && !(worst <= check_tol)) {
     ctx->have_gauge = false;
     char buf[160];

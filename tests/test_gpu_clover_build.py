@@ -80,6 +80,31 @@ def test_su3_check_reports_the_deviation(dims, domain, delta):
         lat.close()
 
 
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf, complex(0.1, np.nan)])
+@pytest.mark.parametrize("site", [(0, 0, 0, 0), (7, 3, 2, 1)])
+def test_non_finite_links_fail_the_su3_check(site, value):
+    """The check refuses them at the default tolerance and at a wide one."""
+    from paper_2109_10687_gb300 import binding as B
+    from paper_2109_10687_gb300.lattice import Lattice
+
+    u = random_su3_field((4, 4, 4, 8), 0.3, 4005)
+    u[site + (2, 0, 1)] = value
+    lat = Lattice((4, 4, 4, 8), (2, 2, 2, 2), -1, "chiral")
+    try:
+        for tol in ({}, {"check_tol": 10.0}):
+            with pytest.raises(B.QcdError) as e:
+                lat.set_gauge(u, **tol)
+            assert e.value.code == B.QCD_ERR_ARG
+        lat.set_params(0.12, 1.0)
+        with pytest.raises(B.QcdError) as e:
+            lat.build_clover()
+        assert e.value.code == B.QCD_ERR_STATE
+        lat.set_gauge(random_su3_field((4, 4, 4, 8), 0.3, 4005))  # and the context goes on
+        lat.build_clover()
+    finally:
+        lat.close()
+
+
 def test_non_finite_links_are_refused_by_the_clover_build():
     from paper_2109_10687_gb300 import binding as B
     from paper_2109_10687_gb300.lattice import Lattice
