@@ -4,19 +4,19 @@
 // batch solver.
 //
 // Reductions: every reducing kernel accumulates per thread in float32 (the
-// float64 kernels in float64), combines the threads of a block to float64
-// accuracy and lets the last block to finish sum the per-block partials in
+// float64 kernels in float64), combines the threads of a block to at least
+// float64 accuracy and lets the last block to finish sum the per-block partials in
 // float64 in a fixed order, so results do not depend on scheduling.  Kernels
 // run on a grid (blocks, k) with blockIdx.y = k the right-hand side (or, in a
 // ragged batch, the lattice); a Seg says where element k of a stacked vector
 // lives.
 //
-// The float32 sums of a block's threads are combined in double-float (48
+// The float32 sums of a block's threads are combined in triple-float (72
 // bits): this GPU has two float64 lanes per SM, and a tree of float64 shuffles
 // over every warp took more time than the data on vectors of a few MB (a
 // 32-lattice batch: alpha's dot product 60 us against 19 us for p's update,
-// which moves more bytes; with this form 32 us, omega's 74 -> 26 us, the
-// second update 94 -> 57 us).
+// which moves more bytes; with this form 34 us, omega's 74 -> 27 us, the
+// second update 94 -> 53 us).
 #pragma once
 
 #include "qcd_internal.cuh"
@@ -56,10 +56,33 @@ struct Seg {
 // ---------------------------------------------------------------------------
 // reduction machinery
 // ---------------------------------------------------------------------------
+// A sum of float32 numbers as three of them, a + b + c: the errors of the
+// sums of a are summed in b, those of b in c (the cascaded summation of Ogita,
+// Rump and Oishi, "Accurate sum and dot product", 2005, with K = 3).  The error
+// is of order 2^-72 of the summands' magnitudes, below float64's 2^-53, which
+// two of them (48 bits) would not reach.
+struct Sum3 {
+  float a, b, c;
+  __device__ explicit Sum3(float x) : a(x), b(0.f), c(0.f) {}
+  __device__ Sum3(float a_, float b_, float c_) : a(a_), b(b_), c(c_) {}
+  __device__ __forceinline__ void add(float x) {
+    const df64 s = two_sum(a, x), t = two_sum(b, s.lo);
+    a = s.hi;
+    b = t.hi;
+    c += t.lo;
+  }
+  __device__ __forceinline__ void add(const Sum3& o) {
+    const df64 s = two_sum(a, o.a), t = two_sum(b, o.b), u = two_sum(t.hi, s.lo);
+    a = s.hi;
+    b = u.hi;
+    c += o.c + (t.lo + u.lo);
+  }
+  __device__ __forceinline__ double total() const { return (double)a + ((double)b + (double)c); }
+};
+
 // The sum of sh[0 .. RED_THREADS) by one warp, to float64 accuracy: float32
-// entries in double-float, which falls back to float64 when the sum leaves
-// float32's range (or is not finite), float64 entries in float64.  Lane 0's
-// value counts.
+// entries as Sum3, which falls back to float64 when the sum leaves float32's
+// range (or is not finite), float64 entries in float64.  Lane 0's value counts.
 __device__ __forceinline__ double warp_tree(double d) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
@@ -69,13 +92,14 @@ template <typename T>
 __device__ __forceinline__ double warp_total(const T* sh) {
   const int lane = threadIdx.x & 31;
   if constexpr (sizeof(T) == 4) {
-    df64 s(sh[lane]);
+    Sum3 s(sh[lane]);
 #pragma unroll
-    for (int j = 1; j < RED_THREADS / 32; ++j) s = s + df64(sh[lane + 32 * j]);
+    for (int j = 1; j < RED_THREADS / 32; ++j) s.add(sh[lane + 32 * j]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
-      s = s + df64(__shfl_down_sync(0xffffffffu, s.hi, o), __shfl_down_sync(0xffffffffu, s.lo, o));
-    if (isfinite(__shfl_sync(0xffffffffu, s.hi, 0))) return to_double(s);
+      s.add(Sum3(__shfl_down_sync(0xffffffffu, s.a, o), __shfl_down_sync(0xffffffffu, s.b, o),
+                 __shfl_down_sync(0xffffffffu, s.c, o)));
+    if (isfinite(__shfl_sync(0xffffffffu, s.a, 0))) return s.total();
   }
   double d = sh[lane];
 #pragma unroll
