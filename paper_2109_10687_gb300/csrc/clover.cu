@@ -81,7 +81,8 @@ __device__ M3 prod4(const M3& a, const M3& b, const M3& c, const M3& d) {
 }
 
 // F_mu,nu = (Q - Q^dag) / 8 in float64, for links that need not be SU(3)
-// (and so have no bound): the nine reals of field_strength_fx
+// (and so have no bound) or whose small entries count: the nine reals of
+// field_strength_fx
 __device__ __noinline__ void field_strength(const Geom& g, const LinkPtr<double>& U, const int x[4], int mu, int nu,
                                             double f[9]) {
   auto at = [&](int dm, int dn, int dir) {
@@ -570,8 +571,13 @@ __global__ void links_to_fixed_kernel(const double2* __restrict__ u64, int4* out
 }
 
 // The fixed-point path takes links that set_gauge found to be SU(3) to 1e-9
-// (their entries are bounded by one); any others, which a caller may set by
-// switching that check off, take the float64 products.
+// (their entries are bounded by one) and not near the diagonal anywhere; any
+// others (fields near the identity, and whatever a caller sets with the check
+// switched off) take the float64 products.  24^3 x 48: 3.3 ms in fixed point,
+// 10.1 ms in float64.  Error of the off-diagonal part of 1 + C on links
+// exp(i eps H), fixed point against float64: 4.9e-16 and 4.8e-16 at eps 0.05,
+// 5.0e-16 and 4.8e-16 at 0.02, 2.2e-15 and 4.8e-16 at 1e-3, 2e-12 at 1e-6: in
+// steps of 2^-58 whatever the entries' size.
 void build_clover_launch(qcd_ctx* ctx, cudaStream_t st) {
   const Geom& g = ctx->geom;
   const CloverOut o{ctx->clov64, ctx->cinv64, ctx->clov32, ctx->cinv32, ctx->cinv16, ctx->clovdf,
@@ -585,7 +591,7 @@ void build_clover_launch(qcd_ctx* ctx, cudaStream_t st) {
     kernel<<<blocks, threads, 0, st>>>(args...);
     check_launch();
   };
-  if (ctx->su3_links) {
+  if (ctx->fixed_clover) {
     // scratch: the limbs where 1 + C goes in double-float, the next sites'
     // shares of F where the double-float links go once the clover term is built
     int4* ufx = reinterpret_cast<int4*>(ctx->clovdf);

@@ -312,10 +312,30 @@ __device__ __forceinline__ double su3_deviation_fx(const double* in, unsigned lo
   return (double)worst * (1.0 / (double)one);
 }
 
+// Entries so small that fixed point (absolute steps of 2^-58) would keep fewer
+// of their bits than float64 does: a link near the identity (imaginary parts of
+// the diagonal and off-diagonal entries below 2^-6, not all zero) or near the
+// diagonal matrices (off-diagonal entries below 2^-8, not all zero).  By the
+// upper halves of the bit patterns.
+__device__ __forceinline__ bool link_near_diagonal(const double* in) {
+  unsigned off = 0, dia = 0;
+#pragma unroll
+  for (int e = 0; e < 18; ++e) {
+    const unsigned h = (unsigned)__double2hiint(in[e]) & 0x7FFFFFFFu;
+    if (e / 2 % 4) off = max(off, h);
+    else if (e & 1) dia = max(dia, h);
+  }
+  constexpr unsigned k2m6 = 0x3F900000u, k2m8 = 0x3F700000u;
+  return off ? off < k2m8 || max(off, dia) < k2m6 : dia && dia < k2m6;
+}
+
 // canonical gauge field -> internal float64 / float32 / float16 links and
 // float32 two-row links, with an SU(3) check that records the worst deviation
 // in bad[0] (as the bit pattern of a non-negative double, so integer atomicMax
 // orders it; NaN entries drop out of it) and any non-finite entry in bad[1].
+// bad[2]: some site has two near-diagonal links.  The leaves of F in a plane
+// through a site include the site's links in both directions of the plane, so
+// otherwise no F is a sum over near-diagonal links only.
 // A block takes 32 sites in internal order, a thread one link: the canonical
 // reads (576 contiguous bytes a site) go through shared memory, and every
 // write is one stream over consecutive sites.  Latency bounds it (loads,
@@ -331,10 +351,12 @@ __global__ void __launch_bounds__(GI_THREADS, 6) gauge_import_kernel(Geom g, con
   __shared__ double buf[GI_SITES * GI_ROW];
   __shared__ unsigned canon[GI_SITES];
   __shared__ unsigned long long s_worst;
+  __shared__ int s_near[GI_SITES], s_two;
   const long long n0 = blockIdx.x * (long long)GI_SITES;
   const int live = (int)min((long long)GI_SITES, g.vol - n0);
   const int site = threadIdx.x & (GI_SITES - 1), mu = threadIdx.x / GI_SITES;
-  if (threadIdx.x == 0) s_worst = 0;
+  if (threadIdx.x == 0) s_worst = s_two = 0;
+  if (mu == 0) s_near[site] = 0;
   const long long gid = n0 + (site < live ? site : 0);
   const int s = (int)(gid & (g.vd - 1));
   int lex = (int)(gid >> g.logvd);
@@ -372,9 +394,13 @@ __global__ void __launch_bounds__(GI_THREADS, 6) gauge_import_kernel(Geom g, con
       u32c[cbase + ((size_t)q << g.logvd)] =
           make_float4((float)in[4 * q], (float)in[4 * q + 1], (float)in[4 * q + 2], (float)in[4 * q + 3]);
     atomicMax(&s_worst, (unsigned long long)__double_as_longlong(su3_deviation_fx(in, bad + 1)));
+    if (link_near_diagonal(in) && atomicAdd(&s_near[site], 1) == 1) s_two = 1;
   }
   __syncthreads();
-  if (threadIdx.x == 0) atomicMax(bad, s_worst);
+  if (threadIdx.x == 0) {
+    atomicMax(bad, s_worst);
+    if (s_two) atomicExch(bad + 2, 1ull);
+  }
 }
 
 }  // namespace qcd
@@ -548,13 +574,13 @@ extern "C" int qcd_set_gauge(qcd_ctx* ctx, const double* U, int on_device, doubl
     src = tmp;
   }
   unsigned long long* bad = (unsigned long long*)ctx->d_status + 1;
-  QCD_CUDA_CHECK(cudaMemsetAsync(bad, 0, 2 * sizeof(unsigned long long), st));
+  QCD_CUDA_CHECK(cudaMemsetAsync(bad, 0, 3 * sizeof(unsigned long long), st));
   {
     LaunchScope ls(ctx, QCD_KC_OTHER, st);
     gauge_import_kernel<<<grid_for(g.vol, GI_SITES), GI_THREADS, 0, st>>>(g, src, ctx->u64, ctx->u32, ctx->u16, ctx->u32c, bad);
     check_launch();
   }
-  unsigned long long hbad[2] = {0, 0};
+  unsigned long long hbad[3] = {0, 0, 0};
   QCD_CUDA_CHECK(cudaMemcpyAsync(hbad, bad, sizeof(hbad), cudaMemcpyDeviceToHost, st));
   QCD_CUDA_CHECK(cudaStreamSynchronize(st));
   if (tmp) cudaFree(tmp);
@@ -563,6 +589,7 @@ extern "C" int qcd_set_gauge(qcd_ctx* ctx, const double* U, int on_device, doubl
   ctx->have_gauge = true;
   ctx->have_clover = false;
   ctx->su3_links = worst <= 1e-9 && hbad[1] == 0;
+  ctx->fixed_clover = ctx->su3_links && hbad[2] == 0;
   // NaN entries drop out of the worst deviation (fmax), so they have a word of their own
   if (check_tol > 0 && hbad[1]) {
     ctx->have_gauge = false;

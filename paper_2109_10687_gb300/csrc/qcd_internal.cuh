@@ -701,6 +701,7 @@ struct qcd_ctx {
   __half2* u16 = nullptr;
   float4* u32c = nullptr;          // float32 links as their first two rows (12 reals, three float4)
   bool su3_links = false;          // every link is SU(3) to 1e-9: the third row follows from the first two
+  bool fixed_clover = false;       // F of the clover term in fixed point: SU(3) links, not near the diagonal
   int link12 = -1;                 // float32 D with links as 12 reals: -1 when SU(3), 0 never, 1 always
   double2* clov64 = nullptr;     // 1 + C
   float4* clov32 = nullptr;

@@ -80,6 +80,57 @@ def test_su3_check_reports_the_deviation(dims, domain, delta):
         lat.close()
 
 
+def _near_fields():
+    """Links near the identity, near the diagonal matrices, and rough ones with
+    a patch of each: (name, U, sites to compare)."""
+    dims = (8, 8, 8, 8)
+    everywhere = np.ones((8, 8, 8, 8), dtype=bool)
+    for eps in (0.05, 0.01, 1e-3, 1e-6, 1e-9):
+        yield "identity_%g" % eps, random_su3_field(dims, eps, 4006), everywhere
+    theta = np.random.default_rng(4007).uniform(-1, 1, size=(8, 8, 8, 8, 4, 3))
+    theta -= theta.mean(axis=-1, keepdims=True)
+    near = random_su3_field(dims, 1e-5, 4008)
+    yield "diagonal_1e-5", np.exp(1j * theta)[..., None] * near, everywhere
+    yield "diagonal_small", np.exp(1e-6j * theta)[..., None] * np.eye(3), everywhere
+    patch = random_su3_field(dims, 0.4, 4009)
+    patch[2:5, 1:4, 3:6, 4:7] = random_su3_field(dims, 1e-6, 4006)[2:5, 1:4, 3:6, 4:7]
+    inner = np.zeros((8, 8, 8, 8), dtype=bool)
+    inner[3, 2, 4, 5] = True  # every leaf of this site lies in the patch
+    yield "patch", patch, inner
+
+
+@pytest.mark.parametrize("name,u,sites", list(_near_fields()), ids=lambda v: v if isinstance(v, str) else "")
+def test_small_entries_of_the_clover_term_keep_their_bits(name, u, sites):
+    """The off-diagonal part of 1 + C, relative to itself: products of float64
+    numbers near one and small ones keep the small ones' relative accuracy
+    (5e-16 measured in float64, against the oracle's own 2e-16)."""
+    from oracle.dirac import clover_term
+    from oracle.gamma import gamma_chiral
+    from paper_2109_10687_gb300.lattice import Lattice
+
+    c = clover_term(u, 0.125, 1.0, gamma_chiral())
+    # colour-diagonal entries and the others, each relative to their own norm
+    kinds = {"colour": ~np.kron(np.eye(3), np.ones((4, 4))).astype(bool),
+             "spin": np.kron(np.eye(3), np.ones((4, 4)) - np.eye(4)).astype(bool)}
+    lat = Lattice((8, 8, 8, 8), (4, 4, 4, 4), -1, "chiral")
+    try:
+        lat.set_gauge(u)
+        lat.set_params(0.125, 1.0)
+        lat.build_clover()
+        m = np.empty(c.shape, dtype=complex)
+        for j in range(12):
+            psi = np.zeros(c.shape[:4] + (12,), dtype=complex)
+            psi[..., j] = 1
+            out = lat.apply_clover(psi.reshape(c.shape[:4] + (3, 4)), "double")
+            m[..., :, j] = (out.detach().cpu().numpy() if hasattr(out, "detach") else out).reshape(c.shape[:4] + (12,))
+    finally:
+        lat.close()
+    for kind, mask in kinds.items():
+        ref = c[sites][..., mask]
+        if np.abs(ref).max() > 0:
+            assert np.linalg.norm(m[sites][..., mask] - ref) <= 2e-15 * np.linalg.norm(ref), (name, kind)
+
+
 @pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf, complex(0.1, np.nan)])
 @pytest.mark.parametrize("site", [(0, 0, 0, 0), (7, 3, 2, 1)])
 def test_non_finite_links_fail_the_su3_check(site, value):
