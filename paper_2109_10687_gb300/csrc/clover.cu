@@ -426,8 +426,12 @@ __global__ void __launch_bounds__(FS_THREADS, 3) field_strength_kernel(Geom g, c
 }
 
 // float64 rounded to float32 on the bit fields (conversions would queue on
-// the float64 pipe; results below float32's normal range become zero)
-__device__ __forceinline__ float to_float(double d) { return df64_from_double_scaled(d, 0).hi; }
+// the float64 pipe); what lies outside float32's normal range is converted
+__device__ __forceinline__ float to_float(double d) {
+  const unsigned e = ((unsigned)__double2hiint(d) >> 20) & 0x7FFu;
+  if (e != 0 && e - (1023 - 126) >= 254) return (float)d;
+  return df64_from_double_scaled(d, 0).hi;
+}
 
 // F of a plane at a site, fixed point: the site's own share and the one that
 // the thread of the site before it along mu left

@@ -131,6 +131,33 @@ def test_small_entries_of_the_clover_term_keep_their_bits(name, u, sites):
             assert np.linalg.norm(m[sites][..., mask] - ref) <= 2e-15 * np.linalg.norm(ref), (name, kind)
 
 
+@pytest.mark.parametrize("inverse", [False, True])
+@pytest.mark.parametrize("eps", [3e-37, 1e-38, 1e-41, 1e-44])
+def test_float32_copies_below_the_normal_range(eps, inverse):
+    """Off-diagonal entries of 1 + C and C_inv around float32's smallest normal
+    number: the float32 copies are the float64 ones rounded (to 2^-24, or half
+    of the smallest subnormal 2^-149)."""
+    from paper_2109_10687_gb300.lattice import Lattice
+
+    dims = (4, 4, 4, 4)
+    h = (random_su3_field(dims, 1e-3, 4010) - np.eye(3)) * (1e3 * eps)
+    h = (h - np.conj(np.swapaxes(h, -1, -2))) / 2  # anti-Hermitian: 1 + h is SU(3) to rounding
+    lat = Lattice(dims, (2, 2, 2, 2), -1, "chiral")
+    try:
+        lat.set_gauge(np.eye(3) + h)
+        lat.set_params(0.125, 1.0)
+        lat.build_clover()
+        psi = np.zeros((4, 4, 4, 4, 3, 4), dtype=complex)
+        psi[..., 1, 2] = 1
+        double, single = (lat.apply_clover(psi, prec, inverse=inverse) for prec in ("double", "single"))
+        double, single = (a.detach().cpu().numpy() if hasattr(a, "detach") else a for a in (double, single))
+    finally:
+        lat.close()
+    assert 0 < np.abs(double[..., 0, 2]).min() < 10 * eps
+    for a, b in ((single.real, double.real), (single.imag, double.imag)):
+        assert np.all(np.abs(a - b) <= 2.0**-24 * np.abs(b) + 2.0**-150)
+
+
 @pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf, complex(0.1, np.nan)])
 @pytest.mark.parametrize("site", [(0, 0, 0, 0), (7, 3, 2, 1)])
 def test_non_finite_links_fail_the_su3_check(site, value):
