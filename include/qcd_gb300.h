@@ -350,7 +350,11 @@ int qcd_batch_set_shared(qcd_batch* batch, int enable);
  * skip the two solves; otherwise they are solved with params (when both are
  * needed and params->outer_restart = 0, as the two right-hand sides b and
  * gamma_5 eta of one batched solve).
- * grad_U layout: canonical gauge layout. */
+ * grad_U layout: canonical gauge layout.
+ * Scratch: 192 B per site for every canonical source and solution that the
+ * call solves for, and 624 B per site for grad_U (192 with c_SW = 0); 1392 B
+ * per site with both solves.  The context keeps up to 128 MB of it for the next
+ * call (freed in qcd_destroy); a call that needs more frees it on return. */
 int qcd_grad(qcd_ctx* ctx, const double* eta, const double* b, const double* x,
              const double* lam, double* grad_b, double* grad_U, int project,
              const qcd_solve_params* params, void* stream);

@@ -301,6 +301,8 @@ __global__ void gamma5_canonical_kernel(long long vol, double* f, int paper_basi
   }
 }
 
+constexpr size_t GRAD_KEEP = size_t(128) << 20;
+
 }  // namespace qcd
 
 using namespace qcd;
@@ -326,20 +328,29 @@ extern "C" int qcd_grad(qcd_ctx* ctx, const double* eta, const double* b, const 
     const int with_clover = ctx->csw != 0.0;
     // one solve of two right-hand sides when both x and lambda are missing
     const bool both = !x && !lam && P.outer_restart == 0;
-    // Scratch in one buffer kept in the context (cudaMalloc and cudaFree of its
-    // parts took 0.5 ms of a 16^4 call): canonical sources and solutions of
-    // the solves, then the float32 fields and V of the force.
+    // Scratch in one buffer: canonical sources and solutions of the solves,
+    // then the float32 fields and V of the force.  Up to GRAD_KEEP bytes stay
+    // in the context (cudaMalloc and cudaFree of the parts took 0.5 ms of 5.8
+    // at 16^4, 91 MB); a larger buffer, whose call takes longer, is given back.
     const size_t n_src = both ? 2 : (lam ? 0 : 1), n_sol = both ? 2 : (x ? 0 : 1) + (lam ? 0 : 1);
     const size_t force_bytes = grad_U ? 2 * b32 + (with_clover ? (size_t)g.vol * 54 * sizeof(float2) : 0) : 0;
     const size_t need = (n_src + n_sol) * cbytes + force_bytes;
-    if (need > ctx->grad_bytes) {
+    struct Scratch {  // of this call only
+      void* p = nullptr;
+      ~Scratch() {
+        if (p) cudaFree(p);
+      }
+    } own;
+    if (need > GRAD_KEEP) {
+      QCD_CUDA_CHECK(cudaMalloc(&own.p, need));
+    } else if (need > ctx->grad_bytes) {
       if (ctx->grad_buf) QCD_CUDA_CHECK(cudaFree(ctx->grad_buf));
       ctx->grad_buf = nullptr;
       ctx->grad_bytes = 0;
       QCD_CUDA_CHECK(cudaMalloc(&ctx->grad_buf, need));
       ctx->grad_bytes = need;
     }
-    double* src = static_cast<double*>(ctx->grad_buf);
+    double* src = static_cast<double*>(own.p ? own.p : ctx->grad_buf);
     double* sol = src + n_src * fdoubles;
     float4* x32 = reinterpret_cast<float4*>(sol + n_sol * fdoubles);
     float4* l32 = x32 + b32 / sizeof(float4);

@@ -727,7 +727,7 @@ struct qcd_ctx {
   int cl_gen = -1;
   int cl_dom[4] = {0, 0, 0, 0};
   int inject = 0;                  // testing: QCD_INJECT_* fault (host-side, bounded)
-  void* grad_buf = nullptr;        // scratch of qcd_grad, kept between calls
+  void* grad_buf = nullptr;        // scratch of qcd_grad kept between calls, 128 MB at most
   size_t grad_bytes = 0;
   qcd::Workspace* ws = nullptr;
   qcd::Profiler* prof = nullptr;

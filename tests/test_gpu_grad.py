@@ -61,3 +61,34 @@ def test_autograd_function_matches_oracle():
         assert rel_l2(to_np(ut.grad), g_ref) < 1e-5
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("dims,kept", [((8, 8, 8, 16), True), ((16, 16, 16, 32), False)])
+def test_scratch_beyond_the_bound_is_given_back(dims, kept):
+    """Both solves and the force take 1392 B per site: 11 MB, which the context
+    keeps, and 182 MB, which it does not."""
+    from paper_2109_10687_gb300 import binding as B
+
+    p = Problem(dims, (4, 4, 4, 4), eps=0.2, kappa=0.1, csw=1.0, seed=3200, oracle=False)
+    try:
+        vol = int(np.prod(dims))
+        need = 1392 * vol
+        assert (need <= 128 << 20) == kept
+        b_t = torch.view_as_real(torch.from_numpy(p.source(3201, 2))).cuda().contiguous()
+        x = torch.empty_like(b_t)
+        gb = torch.empty_like(b_t[0])
+        gu = torch.empty(p.lat.site_shape + (4, 3, 3, 2), dtype=torch.float64, device="cuda")
+        params = B.qcd_solve_params_default()
+        B.qcd_solve(p.lat.ctx, x, b_t, 2, params)  # the workspace and its graphs are there
+        B.qcd_grad(p.lat.ctx, b_t[0], b_t[1], gb, None, x=x[1], lam=x[0], params=params)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        held = []
+        for _ in range(2):
+            B.qcd_grad(p.lat.ctx, b_t[0], b_t[1], gb, gu, params=params)
+            held.append(before - torch.cuda.mem_get_info()[0])
+        assert held[0] == held[1]  # nothing is left behind by each call
+        # allocations are rounded up to 2 MB
+        assert held[0] <= (need + (2 << 20) if kept else 2 << 20)
+    finally:
+        p.close()
