@@ -773,6 +773,7 @@ extern "C" int qcd_device_status(qcd_ctx* ctx, int* status, int reset, void* str
 
 extern "C" int qcd_test_inject(qcd_ctx* ctx, int what) {
   if (!ctx || what < QCD_INJECT_NONE || what > QCD_INJECT_HALO_WAIT) return QCD_ERR_ARG;
+  if (what != ctx->inject) workspace_reset_graphs(ctx);  // captured without it, or with it
   ctx->inject = what;
   return QCD_OK;
 }

@@ -181,6 +181,7 @@ extern "C" int qcd_link_format(const qcd_ctx* ctx, int* reals) {
 
 extern "C" int qcd_set_sap_shape(qcd_ctx* ctx, int shape) {
   if (!ctx || shape < -1 || shape > 4) return QCD_ERR_ARG;
+  if (shape != ctx->sap_shape) workspace_reset_graphs(ctx);  // captured with the other shape
   ctx->sap_shape = shape;
   return QCD_OK;
 }

@@ -154,6 +154,39 @@ def test_algorithm5_iterates_match_oracle(c1):
     assert rel_l2(to_np(x), bn * x_or) < 2e-5
 
 
+@pytest.mark.parametrize("use_graph", [1, 2])
+def test_a_captured_loop_follows_the_shape_and_the_hook(c1, c1_ref, use_graph):
+    """A solve replays its inner loop from the graphs of an earlier one; after
+    qcd_set_sap_shape or qcd_test_inject it is captured anew.  Shape 0 launches
+    2 (n_sap + 1) kernels per M_SAP, shape 3 one."""
+    from paper_2109_10687_gb300 import binding as B
+    b, _ = c1_ref
+    ctx = c1.lat.ctx
+    args = dict(tol=1e-10, sap_prec="half_gauge", inner_tol=1e-5, use_graph=use_graph)
+
+    def launches():
+        c1.lat.solve(b, **args)  # captured, if it has to be
+        n0 = B.qcd_launch_count(ctx)
+        c1.lat.solve(b, **args)
+        return B.qcd_launch_count(ctx) - n0
+
+    try:
+        B.qcd_set_sap_shape(ctx, 0)
+        steps = launches()
+        B.qcd_set_sap_shape(ctx, 3)
+        assert launches() < steps / 2
+        B.qcd_test_inject(ctx, B.INJECT_STAGING_WAIT)
+        # one iteration: every M_SAP in it waits for its half second
+        _, rc, _ = c1.lat.solve(b, raise_on_error=False, max_outer=1, max_inner=1, **args)
+        assert rc == B.QCD_ERR_TIMEOUT
+    finally:
+        B.qcd_test_inject(ctx, B.INJECT_NONE)
+        B.qcd_device_status(ctx, reset=True)
+        B.qcd_set_sap_shape(ctx, -1)
+    _, rc, _ = c1.lat.solve(b, **args)
+    assert rc == 0
+
+
 @pytest.mark.parametrize("use_graph", [0, 2])
 def test_batched_point_sources(c1, use_graph):
     """Several spin-colour point sources in one batched solve (the device-side
