@@ -426,6 +426,15 @@ int qcd_link_format(const qcd_ctx* ctx, int* reals);
  * L1.  QCD_ERR_ARG for other values. */
 int qcd_set_sap_shape(qcd_ctx* ctx, int shape);
 
+/* The SAP kernel with four threads per site (4^4 domains, a domain a cluster of
+ * four CTAs), for lattices with too few domains to fill the GPU: -1 (default)
+ * the autotuner tries it beside the shapes of qcd_set_sap_shape while the
+ * domains of a colour times the right-hand sides are few; 0 never; 1 always,
+ * unless qcd_set_sap_shape fixes a shape or a hook of qcd_test_inject is set
+ * (it has none of the waits that the hooks concern).  The same M_SAP bit for
+ * bit.  QCD_ERR_ARG for other values. */
+int qcd_set_sap_split(qcd_ctx* ctx, int mode);
+
 /* Autotuner over SAP domain shapes, by time to solution.  The domain shape
  * fixes a context's field layout, so for each candidate this creates a
  * temporary context (dims, domain = candidate, bc_t, basis as qcd_create),

@@ -84,6 +84,7 @@ _SIGS = {
     "qcd_launch_count": (_I, [_P, ctypes.POINTER(ctypes.c_longlong)]),
     "qcd_set_tuning": (_I, [_P, _I]),
     "qcd_set_sap_shape": (_I, [_P, _I]),
+    "qcd_set_sap_split": (_I, [_P, _I]),
     "qcd_set_link_compression": (_I, [_P, _I]),
     "qcd_link_format": (_I, [_P, ctypes.POINTER(ctypes.c_int)]),
     "qcd_set_sap_domain": (_I, [_P, ctypes.POINTER(ctypes.c_int)]),
@@ -359,6 +360,11 @@ def qcd_set_sap_shape(ctx, shape):
     """SAP block-kernel shape for 4^4 domains: -1 autotuned, 0 one site per
     thread, 1 two sites per thread."""
     return check(ctx, lib().qcd_set_sap_shape(ctx, int(shape)))
+
+
+def qcd_set_sap_split(ctx, mode):
+    """The SAP kernel with four threads per site on 4^4 domains: -1 autotuned, 0 never, 1 always."""
+    return check(ctx, lib().qcd_set_sap_split(ctx, int(mode)))
 
 
 def qcd_measure_fp32_peak(ctx, stream=None):

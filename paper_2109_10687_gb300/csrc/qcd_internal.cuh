@@ -719,6 +719,7 @@ struct qcd_ctx {
   void* st_clov32 = nullptr;
   int* flow_state = nullptr;       // one-launch M_SAP: 2 counters, then one flag per domain (zero at rest)
   int sap_shape = -1;              // SAP block-kernel shape: -1 autotuned, else an index of the shapes
+  int sap_split = -1;              // four threads per site on 4^4 domains: -1 autotuned, 0 never, 1 always
   bool sap_general = false;        // SAP on domains sap_dom, independent of the storage blocking
   int sap_dom[4] = {0, 0, 0, 0};
   int clover_gen = 0;              // counts clover builds (staging copies follow it)

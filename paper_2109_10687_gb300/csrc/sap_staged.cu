@@ -1119,7 +1119,9 @@ static void staged_sequence(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, SIO x, 
                                           v == 2 && nrhs > 1);
   };
   int v = ctx->sap_shape;
-  if (v < 0) {
+  if (v < 0 && ctx->sap_split == 1 && ctx->inject == QCD_INJECT_NONE) {
+    v = kSplitShape;
+  } else if (v < 0) {
     const Geom& g = ctx->geom;
     char key[128];
     std::snprintf(key, sizeof key, "sap_staged_%s L%dx%dx%dx%d nrhs%d n_sap%d n_jac%d",
@@ -1143,7 +1145,7 @@ static void staged_sequence(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, SIO x, 
     if ((long long)g.nhalf * nrhs <= kSplitItems) add(kSplitShape);
     v = cand[tune_pick(ctx, key, nc, names, [&](int c) { run(cand[c]); }, st)];
     // a failure hook concerns the block kernel's waits, which the split one does not have
-    if (v == kSplitShape && ctx->inject != QCD_INJECT_NONE) v = 0;
+    if (v == kSplitShape && (ctx->inject != QCD_INJECT_NONE || ctx->sap_split == 0)) v = 0;
   }
   run(v);
 }

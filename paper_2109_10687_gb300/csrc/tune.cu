@@ -186,6 +186,13 @@ extern "C" int qcd_set_sap_shape(qcd_ctx* ctx, int shape) {
   return QCD_OK;
 }
 
+extern "C" int qcd_set_sap_split(qcd_ctx* ctx, int mode) {
+  if (!ctx || mode < -1 || mode > 1) return QCD_ERR_ARG;
+  if (mode != ctx->sap_split) workspace_reset_graphs(ctx);
+  ctx->sap_split = mode;
+  return QCD_OK;
+}
+
 extern "C" int qcd_tuning_report(qcd_ctx* ctx, char* buf, size_t len) {
   if (!ctx || !buf || len == 0) return QCD_ERR_ARG;
   std::string out;
