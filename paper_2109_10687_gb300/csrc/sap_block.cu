@@ -22,6 +22,7 @@
 // operator reads through L1 and branches, 40 us with four threads per site,
 // 21.4 us here.
 
+#include <algorithm>
 #include <cstdio>
 #include <type_traits>
 
@@ -339,6 +340,20 @@ __global__ void __launch_bounds__(NT, HALF ? 512 / NT : (NT == 64 ? 5 : 256 / NT
   if (live) a.x.store(g, domr, s, xk);
 }
 
+// Shared memory of a launch: what its blocks use, or, if that is more, so much
+// that an SM holds no more of them than an even share.  With room for more, and
+// the next launch's blocks arriving while this one's still run, they pair up on
+// some SMs and leave others idle.  M_SAP (n_sap 4, n_jac 4), float16 links, us
+// without and with: 16^4 on 8x4x4x2 domains 280 and 182, on 2^4 239 and 156;
+// 12x20x12x28 on 2^4 257 and 186; float32, 8^2 16 24 on 2^4, 154 and 104.
+template <bool HALF, int NT>
+static int sb_launch_smem(const qcd_ctx* ctx, long long blocks) {
+  constexpr int SM_BYTES = 228 * 1024, BLOCK_RESERVED = 1024, BLOCK_MAX = 227 * 1024;
+  const long long share = (blocks + ctx->sms - 1) / ctx->sms;
+  const long long pad = SM_BYTES / (share + 1) - BLOCK_RESERVED + 16;  // share + 1 do not fit
+  return (int)std::min<long long>(BLOCK_MAX, std::max<long long>((long long)sb_smem<HALF, NT>(), pad));
+}
+
 // Algorithm 1 as 2 (n_sap + 1) launches, every right-hand side in each.
 // b: the source, also the first sweep's input; x: the result, which holds the
 // iterates of both colours on the way.
@@ -347,9 +362,10 @@ static void block_launches(qcd_ctx* ctx, SIO s, F32Spinor x, F32Spinor b, int nr
                            cudaStream_t st) {
   const long long sites = (long long)ctx->geom.nhalf << ctx->geom.logvd;
   QCD_REQUIRE(sites + NT < (1LL << 31), QCD_ERR_ARG, "SAP: lattice too large");
+  const int blocks = (int)((sites + NT - 1) / NT), smem = sb_launch_smem<HALF, NT>(ctx, (long long)blocks * nrhs);
   // the limit is the current device's, and a process may use several
   QCD_CUDA_CHECK(cudaFuncSetAttribute(sap_block_kernel<HALF, SIO, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sb_smem<HALF, NT>()));
+                                      smem));
   BlockArgs<HALF, SIO> a;
   a.g = ctx->geom;
   a.n_jac = n_jac;
@@ -367,8 +383,7 @@ static void block_launches(qcd_ctx* ctx, SIO s, F32Spinor x, F32Spinor b, int nr
       a.colour = colour;
       a.do_surface = (sweep == 0 && colour == 0) ? 0 : 1;
       LaunchScope ls(ctx, QCD_KC_SAP_BLOCK, st);
-      launch_pdl(sap_block_kernel<HALF, SIO, NT>, dim3((unsigned)((sites + NT - 1) / NT), nrhs), dim3(NT),
-                 sb_smem<HALF, NT>(), st, a);
+      launch_pdl(sap_block_kernel<HALF, SIO, NT>, dim3((unsigned)blocks, nrhs), dim3(NT), smem, st, a);
       check_launch();
     }
   }
