@@ -485,9 +485,12 @@ __global__ void __launch_bounds__(CS_MAX_SLICE, 1) sap_cluster_kernel(ClusterSap
     const bool more = it + 1 < napp;
     if (live) {
       zero(acc);
-      cs_intra_space<0>(xb, sl, S, s, 1, fx, bx, acc);
-      cs_intra_space<1>(xb, sl, S, s, a.sd[0], fy, by, acc);
-      cs_intra_space<2>(xb, sl, S, s, a.sd[0] * a.sd[1], fz, bz, acc);
+      // A direction one site wide has no hops inside: left out where several
+      // are (no halo; 16x4x1x1 domains 645 -> 595 us), else the branches cost
+      // more than they save (16x6x4x3 588 -> 596 us).
+      if (HALO || a.sd[0] > 1) cs_intra_space<0>(xb, sl, S, s, 1, fx, bx, acc);
+      if (HALO || a.sd[1] > 1) cs_intra_space<1>(xb, sl, S, s, a.sd[0], fy, by, acc);
+      if (HALO || a.sd[2] > 1) cs_intra_space<2>(xb, sl, S, s, a.sd[0] * a.sd[1], fz, bz, acc);
       HalfSpinor<float> h, uh;
       if (above) {
         cs_load_half(t_up, S, s, h);
