@@ -151,10 +151,14 @@ constexpr int kNumShapes = 4, kDefaultPair = 3;
 // be several per slot (152 SMs x 4) and few idle halves: at 16^4 with 12
 // right-hand sides (3072 blocks of pairs) A takes 0.0672 ms against 0.0684,
 // but on 8^4 with 4 (64 blocks) 8.4 us against 5.0, and with 3 right-hand
-// sides (a quarter of the pairs' work spare) 0.139 ms against 0.1215.
+// sides (a quarter of the pairs' work spare) 0.139 ms against 0.1215.  With an
+// odd number of them the line lies between 11 and 13 (24^3 x 32, pairs against
+// one per thread: D 0.4145 and 0.4095 ms with 11, 0.4840 and 0.4921 with 13,
+// 0.5514 and 0.5501 with 15, 0.6188 and 0.6344 with 17; A 0.4052 and 0.4037
+// with 11, 0.4728 and 0.4873 with 13).
 static int default_shape(const Geom& g, int nrhs) {
   const int pairs = (nrhs + 1) / 2;
-  const bool few_spare = nrhs % 2 == 0 || nrhs > 20;
+  const bool few_spare = nrhs % 2 == 0 || nrhs > 12;
   return few_spare && (long long)grid_for(g.vol, 128) * pairs >= 5 * 152 * 4 ? kDefaultPair : 0;
 }
 

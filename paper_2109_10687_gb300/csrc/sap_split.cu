@@ -26,7 +26,7 @@
 // (sap_staged.cu), so both give the same M_SAP bit for bit.
 // M_SAP (n_sap 4, n_jac 4): 8^4 on 4^4 domains, float32, 0.134 ms with a thread
 // per site (8 blocks a colour) and 0.105 ms here (32 blocks); 16 8^3 0.134 and
-// 0.121; from 16^2 8^2 on (32 domains a colour) the block kernel is the faster.
+// 0.116; from 16^2 8^2 on (32 domains a colour) the block kernel is the faster.
 // It is bound by shared memory (2.2 KB per site and sweep) in turn with the FMA
 // pipe, between barriers.
 

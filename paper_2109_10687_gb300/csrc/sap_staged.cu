@@ -1089,13 +1089,16 @@ static void flow_sequence(qcd_ctx* ctx, F32Spinor s_first_in32, SIO s, SIO x, F3
 // The last two shapes run the whole of M_SAP in one launch (sap_flow_kernel),
 // the second of them with half of its CTAs starting later, so that the
 // CTAs on one SM load their operators at different times.  While a colour's
-// domains and right-hand sides fit one wave of the block kernel
-// (kSplitItems), the tuner also tries the kernel with four threads per site
-// (sap_split.cu), which wins up to about 16 domains a colour.
+// domains times the right-hand sides are few (kSplitItems), the tuner also tries
+// the kernel with four threads per site (sap_split.cu).  float32 M_SAP (n_sap 4,
+// n_jac 4), us, that kernel and the best other shape: 8 of them (8^4) 105 and
+// 133; 16 (16 8^3) 116 and 134; 24 (8^3 24) 131 and 132; 32 (8^2 16^2) 142 and
+// 132; 64 (8 16^3) 144 and 134; 96 264 and 136; in float16 alike.  So it is
+// tried while it wins or comes close, and not where it takes twice as long.
 static const char* const kSapShapes[] = {"256x1site", "128x2sites", "256x1site_rhs_grid", "one_launch",
                                          "one_launch_staggered", "4threads_per_site"};
 constexpr int kSplitShape = 5;
-constexpr long long kSplitItems = 304;
+constexpr long long kSplitItems = 64;
 constexpr int kFlowStaggerNs = 10000;
 
 template <bool HALF, typename SIO>
