@@ -248,8 +248,9 @@ int qcd_sap_apply_nrhs(qcd_ctx* ctx, void* out, const void* in, int nrhs, int n_
 
 /* ---- BLAS-1 (float32 internal fields, float64 results) --------------- */
 
-/* *result = |a|^2 (host pointer), accumulated per block in float32 and
- * across blocks in float64, in a fixed order (deterministic). */
+/* *result = |a|^2 (host pointer), accumulated per thread in the field's
+ * precision, across threads to float64 accuracy and across blocks in float64,
+ * in a fixed order (deterministic). */
 int qcd_norm2(qcd_ctx* ctx, double* result, const void* a, int prec, int nrhs, void* stream);
 
 /* |a|^2 like qcd_norm2, for callers that must not allocate device memory
